@@ -42,67 +42,129 @@ __global__ void k_validate(int n, const int* __restrict__ rp, const int* __restr
 // ---- levels ---------------------------------------------------------------------------------
 // lower_only: treat only j < i (uplo 0) / j > i (uplo 1) as dependencies and ignore the rest
 // (used for the lower pattern of a general matrix by the factorization).
-__global__ void k_levels(int n, const int* __restrict__ rp, const int* __restrict__ col, int uplo, int* level,
-                         int* nlev, int* status, long long budget) {
+//
+// A warp takes a chunk of 32 consecutive rows of the lower problem, one a lane; chunk c goes to
+// warp c mod W.  What bounds the kernel is the latency of the dependency chain (a poll of a level
+// another warp publishes is an L2 round trip), so a lane's level is published as soon as it is
+// final and not when the chunk is: rows that continue a grid line depend on the chunk before, and
+// a chunk that publishes only as a whole would chain every chunk to its predecessor.
+//  - Dependencies on earlier chunks are polled kLevBatch entries of the row at a time.
+//  - Dependencies inside the chunk: with runs, maximal stretches of lanes each depending on the
+//    lane before it, the levels of a run are l_i = max over j <= i of (e_j + i - j) (e: from the
+//    earlier chunks), one segmented maximum scan of five shuffles; lane i is final when every lane
+//    of its run up to i has all of its e.  Other dependencies on lanes of the same run add nothing
+//    (the run already orders them).  Only a chunk with a dependency on a lane outside the run (a
+//    grid line shorter than a chunk, an entry dropped from a factor) takes the general pass: 32
+//    shuffles in lane order.  Either is done when a lane has just read its last outside level.
+//  - The more warps are resident the more rows are in flight, but the polls of the warps that are
+//    still far from the wavefront delay everyone's: with 64 warps an SM polling continuously one
+//    analysis takes 10 to 300 ms.  So a warp that has not read a single level yet sleeps between
+//    its polls; one that has read some polls continuously.
+// Whole analysis (validation and sort included) of ILU(0) factors, publishing whole chunks / this:
+// 7-point 128^3 (lines of whole chunks) 0.75 / 0.61 ms; 576 Schwarz boxes of 128^3 (lines of 34 rows)
+// 59 / 0.80 ms; ILUT of the 27-point stencil on 100^3 about 80 / 1.4 ms.  One microsecond of sleep:
+// with none 9.7, 160 and 56 ms for 128^3, 127^3 and that ILUT factor, with 1 us 0.61, 1.59 and 1.39, with
+// 2 us 0.87, 1.44 and 1.11; with 32 warps an SM and no sleep 0.96, 1.37 and 1.11.
+constexpr int kLevBatch = 4;
+constexpr int kLevFarNs = 1000;
+
+__global__ void __launch_bounds__(256, 8) k_levels(int n, const int* __restrict__ rp, const int* __restrict__ col, int uplo,
+                                                int* level, int* nlev, int* status, long long budget) {
+    const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     const int chunks = (n + 31) >> 5;
+    const unsigned below = (2u << lane) - 1u;  // this lane and those before it
     int mymax = 0;
-    // A chunk is 32 consecutive rows of the lower problem.  A dependency inside the chunk is on an
-    // earlier lane and is resolved with shuffles (one pass over the lanes in order: a lane's level
-    // is final once every lower lane has been broadcast); only dependencies on earlier chunks are
-    // read from memory, polled up to 8 at a time.
     for (int c = gw; c < chunks; c += nw) {
-        const int base = c << 5;
-        const int t = base + lane;
-        int lev = 0;
-        unsigned intra = 0;  // lanes of this chunk that this row depends on
-        int i = 0;
-        if (t < n) {
-            i = uplo ? n - 1 - t : t;
-            const int a = rp[i], b = rp[i + 1];
-            const int* wl[8];
-            int nwait = 0;
-            for (int p = a; p < b; ++p) {
-                const int j = __ldg(col + p);
-                const bool dep = uplo ? (j > i) : (j < i);
-                if (!dep || j < 0 || j >= n) continue;
+        const int base = c << 5, t = base + lane;
+        const int i = uplo ? n - 1 - t : t;
+        int lev = 0, p = 0, b = 0, cc[kLevBatch];
+        unsigned intra = 0, pend = 0;  // lanes of this chunk this row depends on; slots of cc still to be read
+        auto load_batch = [&]() {
+#pragma unroll
+            for (int q = 0; q < kLevBatch; ++q) cc[q] = p + q < b ? __ldg(col + p + q) : -1;
+#pragma unroll
+            for (int q = 0; q < kLevBatch; ++q) {
+                const int j = cc[q];
+                if (j < 0 || j >= n || !(uplo ? j > i : j < i)) continue;
                 const int tj = uplo ? n - 1 - j : j;  // its position in the lower problem, < t
-                if (tj >= base) {
-                    intra |= 1u << (tj - base);
-                    continue;
-                }
-                wl[nwait++] = level + j;
-                if (nwait == 8 || p + 1 == b) {
-                    int lv[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) lv[q] = q < nwait ? (int)ld_relaxed_u32(wl[q]) : 0;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (q < nwait) {
-                            const int lj = lv[q] == kSentI ? wait_i32(wl[q], status, budget) : lv[q];
-                            lev = max(lev, lj + 1);
-                        }
-                    nwait = 0;
-                }
+                if (tj >= base) intra |= 1u << (tj - base);
+                else pend |= 1u << q;
             }
-            if (nwait) {
-                for (int q = 0; q < nwait; ++q) lev = max(lev, wait_i32(wl[q], status, budget) + 1);
-            }
-        }
-#pragma unroll
-        for (int d = 0; d < 32; ++d) {
-            const int ld = __shfl_sync(0xffffffffu, lev, d);
-            if ((intra >> d) & 1u) lev = max(lev, ld + 1);
-        }
+        };
         if (t < n) {
-            publish_i32(level + i, lev);
-            mymax = max(mymax, lev + 1);
+            p = __ldg(rp + i);
+            b = __ldg(rp + i + 1);
+            load_batch();
+        }
+        unsigned ready = 0u, out = 0u;  // lanes whose outside levels are all read; lanes published
+        bool first = true;
+        const long long t0 = clock64();
+        unsigned failed = 0u;
+        for (unsigned it = 1;; ++it) {
+            if (it > 1u && !__any_sync(full, lev > 0)) __nanosleep(kLevFarNs);  // nothing has arrived: far ahead
+            int v[kLevBatch];
+#pragma unroll
+            for (int q = 0; q < kLevBatch; ++q)
+                if ((pend >> q) & 1u) v[q] = (int)ld_relaxed_u32(level + cc[q]);
+#pragma unroll
+            for (int q = 0; q < kLevBatch; ++q)
+                if (((pend >> q) & 1u) && v[q] != kSentI) {
+                    lev = max(lev, v[q] + 1);
+                    pend &= ~(1u << q);
+                }
+            if (pend == 0u && p + kLevBatch < b) {
+                p += kLevBatch;
+                load_batch();
+            }
+            const unsigned now = __ballot_sync(full, pend == 0u && p + kLevBatch >= b);
+            if (now != ready || first) {
+                ready = now;
+                first = false;
+                const unsigned starts = __ballot_sync(full, lane == 0 || !((intra >> (lane - 1)) & 1u));
+                const int rs = 31 - __clz((int)(starts & below));
+                const unsigned mine = below & ~((1u << rs) - 1u);  // the run up to this lane
+                int l;
+                bool fin;
+                if (!__any_sync(full, ((ready >> lane) & 1u) && (intra & ~mine))) {
+                    l = lev - lane;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int u = __shfl_up_sync(full, l, o);
+                        if (lane - o >= rs) l = max(l, u);
+                    }
+                    l += lane;
+                    fin = (ready & mine) == mine;
+                } else {
+                    l = lev | (((ready >> lane) & 1u) ? 0 : (int)0x80000000);  // sign: not final
+#pragma unroll
+                    for (int d = 0; d < 32; ++d) {
+                        const int u = __shfl_sync(full, l, d);
+                        if ((intra >> d) & 1u) l = u < 0 ? (int)0x80000000 : l < 0 ? l : max(l, u + 1);
+                    }
+                    fin = l >= 0;
+                }
+                if (fin && !((out >> lane) & 1u) && t < n) {
+                    publish_i32(level + i, l);
+                    mymax = max(mymax, l + 1);
+                }
+                out = __ballot_sync(full, fin);
+                if (out == full) break;
+            } else if ((it & 63u) == 0u) {
+                const bool give_up = clock64() - t0 > budget || failed != 0u;
+                if (__any_sync(full, give_up)) {  // every wait of the kernel ends: the levels are void
+                    record(status, HEC_ERR_TIMEOUT);
+                    pend = 0u;
+                    p = b;
+                }
+                failed = ld_relaxed_u32(status);
+            }
         }
     }
 #pragma unroll
-    for (int o = 16; o; o >>= 1) mymax = max(mymax, __shfl_xor_sync(0xffffffffu, mymax, o));
+    for (int o = 16; o; o >>= 1) mymax = max(mymax, __shfl_xor_sync(full, mymax, o));
     if (lane == 0 && mymax) atomicMax(nlev, mymax);
 }
 
