@@ -25,14 +25,26 @@ void free_levels(hec_levels* lv);
 
 namespace {
 
+// diagonal positions; code[2] and code[3] receive the longest row and the most pivots in a row
 __global__ void k_find_diag(int n, const int* __restrict__ rp, const int* __restrict__ col, int* dg, int* code) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int d = -1;
-    for (int p = rp[i]; p < rp[i + 1]; ++p)
-        if (col[p] == i) d = p;
-    dg[i] = d;
-    if (d < 0) atomicCAS(code, 0, HEC_ERR_MISSING_DIAG);
+    int len = 0, npiv = 0;
+    if (i < n) {
+        const int a = rp[i], e = rp[i + 1];
+        int d = -1;
+        for (int p = a; p < e; ++p)
+            if (col[p] == i) d = p;
+        dg[i] = d;
+        if (d < 0) atomicCAS(code, 0, HEC_ERR_MISSING_DIAG);
+        len = e - a;
+        npiv = d - a;
+    }
+    len = __reduce_max_sync(0xffffffffu, len);
+    npiv = __reduce_max_sync(0xffffffffu, npiv);
+    if ((threadIdx.x & 31) == 0) {
+        if (len > code[2]) atomicMax(code + 2, len);
+        if (npiv > code[3]) atomicMax(code + 3, npiv);
+    }
 }
 
 // lu holds A's values on the pattern; on return the factors in place.  done[] zeroed.
@@ -124,6 +136,173 @@ __global__ void __launch_bounds__(kIluWarps * 32) k_ilu_numeric(int n, const int
     }
 }
 
+// The elimination for short rows (at most kShortLen entries, kShortPiv of them pivots: the 5- and
+// 7-point patterns): one thread per row, rows in the level order of the lower pattern, U's values
+// their own flags.
+//   What bounds it is the latency of a level: the values of the rows before must be seen and the
+// row's own published.  One warp per row with a completion flag pays an acquire, a dependent load
+// of the pivot row for each pivot, a fence and a release: 11 us a level.  Here the U values are
+// words that start as the sentinel (sync.cuh) and are published one by one with relaxed stores, so a
+// row needs no fence and reads all of its words together: each pivot row's diagonal and its first
+// entry in this row's pattern (further matches, rare, one by one).  Which entries meet the pattern
+// is found before the first wait, and entries that no pivot changes are published then, so that
+// usually only the diagonals are waited for.
+//   The rows of a warp lie scattered in memory: every word polled is a sector of its own, and more
+// than one block an SM (two or three levels of 128^3 in flight) only adds polls.  A warp's rows of
+// one level go together, since an FP64 division costs the same for one lane as for 32; a warp that
+// holds the end of a level and the start of the next takes them in turn.
+//   ilu_factor of the 7-point 128^3 matrix as a whole, warp per row / this: 5.77 / 2.33 ms (3.1 ms with the
+// words of a warp's rows waited for lane by lane, 2.65 ms with every U value published at the end).
+// The operations and their order are those of the kernel above.
+constexpr int kShortLen = 8, kShortPiv = 4;
+constexpr int kShortThreads = 256, kShortBlocks = 1;
+
+// spin on one word (bounded); 0 when the wait gave up
+__device__ __noinline__ double spin_u(const double* p, int* status, long long budget) {
+    return wait_f64(p, status, budget);
+}
+
+__global__ void __launch_bounds__(kShortThreads) k_ilu_short(int n, const int* __restrict__ rp, const int* __restrict__ col,
+                                                             const double* __restrict__ a, const int* __restrict__ dg,
+                                                             const int* __restrict__ order, const int* __restrict__ level,
+                                                             const int* __restrict__ lrp,
+                                                             const int* __restrict__ urp, const int* __restrict__ uci,
+                                                             double* lv, double* uv, int* status, long long budget) {
+    __shared__ double s_val[kShortLen][kShortThreads];
+    __shared__ int s_col[kShortLen][kShortThreads];
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x;
+    const int stride = gridDim.x * kShortThreads;
+    for (int tb = blockIdx.x * kShortThreads + (tid & ~31); tb < n; tb += stride) {
+        const int t = tb + (tid & 31);
+        const bool act = t < n;
+        int i = 0, len = 0, npiv = 0, lev = 0, l0 = 0, u0 = 0;
+        int du[kShortPiv], mu[kShortPiv];         // U word of the pivot's diagonal, of its first match (-1: none)
+        unsigned match[kShortPiv];                // per entry of the pivot row right of its diagonal: 4 bits, the
+                                                  // position of its column in this row (15: not in the pattern)
+        unsigned hit = 0;                         // positions of this row that some pivot changes
+        unsigned pend = 0;                        // words still to be read: bit p the diagonal, bit 4 + p the match
+        double piv[kShortPiv], mv[kShortPiv];
+#pragma unroll
+        for (int p = 0; p < kShortPiv; ++p) {
+            du[p] = 0;
+            mu[p] = -1;
+            match[p] = 0xffffffffu;
+            piv[p] = mv[p] = 0.0;
+        }
+        if (act) {
+            i = __ldg(order + t);
+            const int r0 = __ldg(rp + i);
+            len = __ldg(rp + i + 1) - r0;
+            npiv = __ldg(dg + i) - r0;
+            lev = __ldg(level + i);
+            l0 = __ldg(lrp + i);
+            u0 = __ldg(urp + i);
+#pragma unroll
+            for (int e = 0; e < kShortLen; ++e)
+                if (e < len) {
+                    s_col[e][tid] = __ldg(col + r0 + e);
+                    s_val[e][tid] = __ldg(a + r0 + e);
+                }
+#pragma unroll
+            for (int p = 0; p < kShortPiv; ++p)
+                if (p < npiv) {
+                    const int k = s_col[p][tid];
+                    const int b = __ldg(urp + k), ul = __ldg(urp + k + 1) - b;
+                    du[p] = b;
+                    pend |= 1u << p;
+                    int pos = p + 1;
+#pragma unroll 1
+                    for (int q = 1; q < ul; ++q) {
+                        const int j = __ldg(uci + b + q);
+                        while (pos < len && s_col[pos][tid] < j) ++pos;
+                        if (pos < len && s_col[pos][tid] == j) {
+                            hit |= 1u << pos;
+                            match[p] = (match[p] & ~(15u << (4 * (q - 1)))) | ((unsigned)pos << (4 * (q - 1)));
+                            if (mu[p] < 0) {
+                                mu[p] = b + q;
+                                pend |= 16u << p;
+                            }
+                        }
+                    }
+                }
+        }
+        // U entries that no pivot changes are final: published before the first wait
+        for (int e = npiv + 1; e < len; ++e)
+            if (!((hit >> e) & 1u)) publish_f64(uv + u0 + e - npiv, s_val[e][tid]);
+        // no entry left of the diagonal is changed by an earlier pivot: the quotients are independent
+        const bool indep = (hit & ((1u << npiv) - 1u)) == 0u;
+        bool todo = act;
+        const long long t0 = clock64();
+        // the warp's rows of its lowest level, then those of the next one
+        while (__any_sync(full, todo)) {
+            const int lowest = __reduce_min_sync(full, todo ? lev : 0x7fffffff);
+            const bool now = todo && lev == lowest;
+            for (unsigned it = 1; __any_sync(full, now && pend != 0u); ++it) {
+                if (now) {
+                    unsigned long long w[2 * kShortPiv];
+#pragma unroll
+                    for (int p = 0; p < kShortPiv; ++p) {
+                        if ((pend >> p) & 1u) w[p] = ld_relaxed_u64(uv + du[p]);
+                        if ((pend >> (4 + p)) & 1u) w[kShortPiv + p] = ld_relaxed_u64(uv + mu[p]);
+                    }
+#pragma unroll
+                    for (int p = 0; p < kShortPiv; ++p) {
+                        if (((pend >> p) & 1u) && w[p] != kSent64) {
+                            piv[p] = __longlong_as_double((long long)w[p]);
+                            pend &= ~(1u << p);
+                        }
+                        if (((pend >> (4 + p)) & 1u) && w[kShortPiv + p] != kSent64) {
+                            mv[p] = __longlong_as_double((long long)w[kShortPiv + p]);
+                            pend &= ~(16u << p);
+                        }
+                    }
+                }
+                if ((it & 63u) == 0u && (clock64() - t0 > budget || ld_relaxed_u32(status) != 0u)) {
+                    record(status, HEC_ERR_TIMEOUT);  // every wait of the kernel ends: the factors are void
+                    pend = 0u;
+                }
+            }
+            if (now) {
+                double lik[kShortPiv];
+#pragma unroll
+                for (int p = 0; p < kShortPiv; ++p) lik[p] = indep && p < npiv ? s_val[p][tid] / piv[p] : 0.0;
+#pragma unroll
+                for (int p = 0; p < kShortPiv; ++p)
+                    if (p < npiv) {
+                        if (piv[p] == 0.0) {
+                            record(status, HEC_ERR_ZERO_PIVOT);
+                            continue;
+                        }
+                        if (!indep) lik[p] = s_val[p][tid] / piv[p];
+                        s_val[p][tid] = lik[p];
+                        if (mu[p] < 0) continue;
+                        int q = mu[p] - du[p];  // its first match, then the others
+                        double u = mv[p];
+                        for (unsigned rest = match[p] >> (4 * (q - 1));;) {
+                            const int pos = (int)(rest & 15u);
+                            s_val[pos][tid] = fma(-lik[p], u, s_val[pos][tid]);
+                            do {
+                                rest = (rest >> 4) | 0xf0000000u;
+                                ++q;
+                            } while ((rest & 15u) == 15u && q < kShortLen);
+                            if (q >= kShortLen) break;
+                            u = spin_u(uv + du[p] + q, status, budget);
+                        }
+                    }
+                const double d = s_val[npiv][tid];
+                if (d == 0.0) record(status, HEC_ERR_ZERO_PIVOT);
+                for (int e = npiv + 1; e < len; ++e)
+                    if ((hit >> e) & 1u) publish_f64(uv + u0 + e - npiv, s_val[e][tid]);
+                publish_f64(uv + u0, d);
+                for (int e = 0; e < npiv; ++e) lv[l0 + e] = s_val[e][tid];
+                lv[l0 + npiv] = 1.0;
+                todo = false;
+            }
+        }
+    }
+}
+
 __global__ void k_split_len(int n, const int* __restrict__ rp, const int* __restrict__ dg, int* llen, int* ulen) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -131,6 +310,8 @@ __global__ void k_split_len(int n, const int* __restrict__ rp, const int* __rest
     ulen[i] = rp[i + 1] - dg[i];
 }
 
+// L and U from the pattern and the factors in place; without `lu` only the columns, and U's values
+// set to the sentinel (k_ilu_short writes the values)
 __global__ void k_split(int n, const int* __restrict__ rp, const int* __restrict__ col, const int* __restrict__ dg,
                         const double* __restrict__ lu, const int* __restrict__ lrp, int* lci, double* lv,
                         const int* __restrict__ urp, int* uci, double* uv) {
@@ -139,14 +320,14 @@ __global__ void k_split(int n, const int* __restrict__ rp, const int* __restrict
     int ql = lrp[i];
     for (int p = rp[i]; p < dg[i]; ++p, ++ql) {
         lci[ql] = col[p];
-        lv[ql] = lu[p];
+        if (lu) lv[ql] = lu[p];
     }
     lci[ql] = i;
-    lv[ql] = 1.0;
+    if (lu) lv[ql] = 1.0;
     int qu = urp[i];
     for (int p = dg[i]; p < rp[i + 1]; ++p, ++qu) {
         uci[qu] = col[p];
-        uv[qu] = lu[p];
+        uv[qu] = lu ? lu[p] : __longlong_as_double((long long)kSent64);
     }
 }
 
@@ -338,8 +519,9 @@ HEC_API hec_status ilu_factor(int n, const int* rowptr, const int* col, const do
         return e;
     };
     const int g = (n + 255) / 256;
-    if ((st = dalloc(&code, 2))) return fail(st);
-    HEC_CUDA(cudaMemsetAsync(code, 0, 2 * sizeof(int), s));
+    // [0] errors of the pattern, [1] of the elimination, [2] longest row, [3] most pivots in a row
+    if ((st = dalloc(&code, 4))) return fail(st);
+    HEC_CUDA(cudaMemsetAsync(code, 0, 4 * sizeof(int), s));
     int hcode = 0;
     long long pnnz = 0;
     // ---- pattern ----
@@ -349,8 +531,6 @@ HEC_API hec_status ilu_factor(int n, const int* rowptr, const int* col, const do
         int h = 0;
         if (n > 0) HEC_CUDA(cudaMemcpy(&h, rowptr + n, sizeof(int), cudaMemcpyDeviceToHost));
         pnnz = h;
-        if ((st = dalloc(&lu, (size_t)pnnz))) return fail(st);
-        HEC_CUDA(cudaMemcpyAsync(lu, val, sizeof(double) * (size_t)pnnz, cudaMemcpyDeviceToDevice, s));
     } else if (k >= 2) {
         if (n > 0) {
             if ((st = iluk_pattern(n, rowptr, col, k, &prp, &pci, &pnnz, s))) return fail(st);
@@ -390,31 +570,13 @@ HEC_API hec_status ilu_factor(int n, const int* rowptr, const int* col, const do
     if ((st = dalloc(&dg, (size_t)n))) return fail(st);
     k_find_diag<<<g, 256, 0, s>>>(n, prp, pci, dg, code);
     count_launch();
-    if ((st = read_code(code, s, &hcode))) return fail(st);
-    if (hcode) return fail(set_error(HEC_ERR_MISSING_DIAG, "ilu_factor: a row has no diagonal entry"));
+    int hc[4] = {0, 0, 0, 0};
+    HEC_CUDA(cudaMemcpyAsync(hc, code, sizeof(hc), cudaMemcpyDeviceToHost, s));
+    HEC_CUDA(cudaStreamSynchronize(s));
+    if (hc[0]) return fail(set_error(HEC_ERR_MISSING_DIAG, "ilu_factor: a row has no diagonal entry"));
     lv = new hec_levels();
     if ((st = compute_levels(n, prp, pci, 0, lv, s))) return fail(st);
-    // ---- numeric elimination in level order ----
-    if ((st = dalloc(&done, (size_t)n))) return fail(st);
-    HEC_CUDA(cudaMemsetAsync(done, 0, sizeof(int) * (size_t)n, s));
-    {
-        const int threads = kIluWarps * 32;
-        int per_sm = max_coop_blocks((const void*)k_ilu_numeric, threads, 0);
-        if (per_sm <= 0) return fail(set_error(HEC_ERR_CUDA, "factor kernel cannot be resident"));
-        int blocks = std::max(1, std::min(per_sm * num_sms(), (n + kIluWarps - 1) / kIluWarps));
-        long long budget = 4000000000LL;
-        int nn = n;
-        int* status = code + 1;
-        void* args[] = {&nn, &prp, &pci, &dg, &lv->iperm, &lu, &done, &status, &budget};
-        HEC_CUDA(cudaLaunchCooperativeKernel((const void*)k_ilu_numeric, dim3(blocks), dim3(threads), args, 0, s));
-        count_launch();
-    }
-    int hs[2] = {0, 0};
-    HEC_CUDA(cudaMemcpyAsync(hs, code, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-    HEC_CUDA(cudaStreamSynchronize(s));
-    if (hs[1] == HEC_ERR_ZERO_PIVOT) return fail(set_error(HEC_ERR_ZERO_PIVOT, "ilu_factor: zero pivot"));
-    if (hs[1]) return fail(set_error((hec_status)hs[1], "ilu_factor: dependency wait timed out"));
-    // ---- split into L (unit lower, diagonal stored) and U ----
+    // ---- L (unit lower, diagonal stored) and U: row pointers and storage ----
     int *llen = nullptr, *ulen = nullptr;
     if ((st = dalloc(&llen, (size_t)n + 1)) || (st = dalloc(&ulen, (size_t)n + 1))) {
         dfree(llen);
@@ -431,15 +593,55 @@ HEC_API hec_status ilu_factor(int n, const int* rowptr, const int* col, const do
     dfree(llen);
     dfree(ulen);
     int ln = 0, un = 0;
-    HEC_CUDA(cudaMemcpy(&ln, L->rowptr + n, sizeof(int), cudaMemcpyDeviceToHost));
-    HEC_CUDA(cudaMemcpy(&un, U->rowptr + n, sizeof(int), cudaMemcpyDeviceToHost));
+    HEC_CUDA(cudaMemcpyAsync(&ln, L->rowptr + n, sizeof(int), cudaMemcpyDeviceToHost, s));
+    HEC_CUDA(cudaMemcpyAsync(&un, U->rowptr + n, sizeof(int), cudaMemcpyDeviceToHost, s));
+    HEC_CUDA(cudaStreamSynchronize(s));
     L->nnz = ln;
     U->nnz = un;
     if ((st = dalloc(&L->col, (size_t)ln)) || (st = dalloc(&L->val, (size_t)ln)) || (st = dalloc(&U->col, (size_t)un)) ||
         (st = dalloc(&U->val, (size_t)un)))
         return fail(st);
-    k_split<<<g, 256, 0, s>>>(n, prp, pci, dg, lu, L->rowptr, L->col, L->val, U->rowptr, U->col, U->val);
-    count_launch();
+    // ---- numeric elimination in level order ----
+    // short rows: thread per row, straight into L and U; longer ones: warp per row, in place, then split
+    const bool shortrows = hc[2] <= kShortLen && hc[3] <= kShortPiv;
+    long long budget = 4000000000LL;
+    int nn = n;
+    int* status = code + 1;
+    if (shortrows) {
+        k_split<<<g, 256, 0, s>>>(n, prp, pci, dg, nullptr, L->rowptr, L->col, L->val, U->rowptr, U->col, U->val);
+        count_launch();
+        const int per_sm = std::min(kShortBlocks, max_coop_blocks((const void*)k_ilu_short, kShortThreads, 0));
+        if (per_sm <= 0) return fail(set_error(HEC_ERR_CUDA, "factor kernel cannot be resident"));
+        const int blocks = std::max(1, std::min(per_sm * num_sms(), (n + kShortThreads - 1) / kShortThreads));
+        const double* av = k == 0 ? val : lu;
+        void* args[] = {&nn, &prp, &pci, &av, &dg, &lv->iperm, &lv->level, &L->rowptr, &U->rowptr, &U->col, &L->val, &U->val, &status,
+                        &budget};
+        HEC_CUDA(cudaLaunchCooperativeKernel((const void*)k_ilu_short, dim3(blocks), dim3(kShortThreads), args, 0, s));
+        count_launch();
+    } else {
+        if (k == 0) {
+            if ((st = dalloc(&lu, (size_t)pnnz))) return fail(st);
+            HEC_CUDA(cudaMemcpyAsync(lu, val, sizeof(double) * (size_t)pnnz, cudaMemcpyDeviceToDevice, s));
+        }
+        if ((st = dalloc(&done, (size_t)n))) return fail(st);
+        HEC_CUDA(cudaMemsetAsync(done, 0, sizeof(int) * (size_t)n, s));
+        const int threads = kIluWarps * 32;
+        int per_sm = max_coop_blocks((const void*)k_ilu_numeric, threads, 0);
+        if (per_sm <= 0) return fail(set_error(HEC_ERR_CUDA, "factor kernel cannot be resident"));
+        int blocks = std::max(1, std::min(per_sm * num_sms(), (n + kIluWarps - 1) / kIluWarps));
+        void* args[] = {&nn, &prp, &pci, &dg, &lv->iperm, &lu, &done, &status, &budget};
+        HEC_CUDA(cudaLaunchCooperativeKernel((const void*)k_ilu_numeric, dim3(blocks), dim3(threads), args, 0, s));
+        count_launch();
+    }
+    int hs[2] = {0, 0};
+    HEC_CUDA(cudaMemcpyAsync(hs, code, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    HEC_CUDA(cudaStreamSynchronize(s));
+    if (hs[1] == HEC_ERR_ZERO_PIVOT) return fail(set_error(HEC_ERR_ZERO_PIVOT, "ilu_factor: zero pivot"));
+    if (hs[1]) return fail(set_error((hec_status)hs[1], "ilu_factor: dependency wait timed out"));
+    if (!shortrows) {
+        k_split<<<g, 256, 0, s>>>(n, prp, pci, dg, lu, L->rowptr, L->col, L->val, U->rowptr, U->col, U->val);
+        count_launch();
+    }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(cuda_error(e, "ilu_factor: split"));
