@@ -5,9 +5,20 @@
 // the p largest magnitudes are kept in the strict lower and in the strict upper part (ties to
 // the smaller column), the diagonal always.  L is unit lower with its 1.0 diagonal stored.
 //
-// GB300 design: one cooperative persistent launch; row i belongs to warp i mod W and a warp
-// takes its rows in increasing order, so the smallest unfinished row can always proceed.  A
-// warp keeps its row as a sorted (column, value) list in shared memory; merging U row k is a
+// GB300 design: one cooperative persistent launch.  The rows are cut into runs, stretches of
+// consecutive rows each with an entry in the column before its own (a grid line, for a stencil).
+// A run belongs to a group of warps, dealt out in turn (run r to group r mod G), and its rows to the
+// group's warps in turn; every warp takes its rows in increasing order, so the smallest unfinished
+// row can always proceed.  A row is tens of microseconds of work for one warp (a few for each
+// pivot), so the time is (rows / rows that can work at once): dealt one by one over all warps, only
+// W consecutive rows are in flight, one plane of a 100^3 grid, whose wavefront keeps 33 of the
+// 9,728 warps busy.  Groups put a dozen planes in flight, and a run held by a group holds back no row
+// (each waits for the row before it anyway), while its warps work on the earlier pivots of the rows
+// ahead.  ILUT(10, 1e-3) of the 27-point stencil on 100^3 / 64^3 and of the 7-point matrix on 100^3:
+// row by row 167.6 / 45.1 / 189.0 ms, groups of 8 warps 45.2 / 17.2 / 37.7 (1 warp 100 / 39.7 / 110,
+// 4 warps 61.4 / 22.2 / 56.2, 16 warps 54.4 / 20.0 / 43.0, 32 warps 147 / 41.5 / 153).  Where there
+// are too few runs to give every group one, the groups grow (31 x 33 x 29: 4.9 / 5.2 ms).
+//   A warp keeps its row as a sorted (column, value) list in shared memory; merging U row k is a
 // warp-parallel binary search plus a ballot-ranked insertion of the fill.  A finished row is
 // written into fixed slots (p strictly lower, 1 + p upper entries) and published with a release
 // store of its U length; a row that needs U row k waits for that flag (acquire, bounded).  The
@@ -46,6 +57,9 @@ struct IlutParams {
     int* status;
     long long budget;
     int cap;       // entries of a row's working list
+    const int* __restrict__ runs;  // [nruns + 1] first row of each run
+    int nruns;
+    int g;         // warps that share a run
 };
 
 __device__ __forceinline__ int ld_acquire_flag(const int* p) {
@@ -167,7 +181,21 @@ __global__ void __launch_bounds__(256) k_ilut(IlutParams P) {
     int* s_newp = wc + 2 * cap;
     const int W = gridDim.x * nwb;
     const int up = P.p + 1;
-    for (int i = blockIdx.x * nwb + wl; i < P.n; i += W) {
+    // the group of P.g warps this warp is in, its place there, the current run's next row of it and its end
+    const int gid = blockIdx.x * nwb + wl;
+    int run = gid / P.g, i = 0, rend = 0;
+    const int place = gid % P.g, groups = W / P.g;
+    if (run >= groups) return;  // the last warps do not fill a group
+    for (;;) {
+        i += P.g;
+        if (i >= rend) {
+            do {  // runs shorter than this warp's place have no row for it
+                if (run >= P.nruns) return;
+                i = __ldg(P.runs + run) + place;
+                rend = __ldg(P.runs + run + 1);
+                run += groups;
+            } while (i >= rend);
+        }
         int cur = 0;
         int* col = wc;
         double* val = wv;
@@ -299,6 +327,23 @@ __global__ void __launch_bounds__(256) k_ilut(IlutParams P) {
     }
 }
 
+// run starts: rows without an entry in the column before their own, and every kRunRows-th row (a
+// longer stretch is a chain however it is cut); kRunWarps is the least size of a group
+constexpr int kRunRows = 4096;
+constexpr int kRunWarps = 8;
+__global__ void k_run_flags(int n, const int* __restrict__ rp, const int* __restrict__ ci, int* flag) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int a = rp[i], b = rp[i + 1];
+    const int at = lower_bound(ci, a, b, i - 1);
+    flag[i] = i % kRunRows == 0 || at == b || ci[at] != i - 1;
+}
+__global__ void k_run_starts(int n, const int* __restrict__ flag, const int* __restrict__ pos, int* runs) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n && flag[i]) runs[pos[i]] = i;
+    if (i == 0) runs[pos[n]] = n;
+}
+
 // CSR of L (kept strict entries, then the unit diagonal) and U (diagonal first) from the slots
 __global__ void k_ilut_rowlen(int n, const int* __restrict__ llen, const int* __restrict__ ulen, int* lrl, int* url) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -343,11 +388,11 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
     HEC_CHECK(validate_csr(n, rowptr, col, -1, s));
     hec_csr *L = new hec_csr(), *U = new hec_csr();
     int *lcol = nullptr, *llen = nullptr, *ucol = nullptr, *ulen = nullptr, *status = nullptr, *lrl = nullptr,
-        *url = nullptr;
+        *url = nullptr, *runs = nullptr;
     double *lval = nullptr, *uval = nullptr;
     auto cleanup = [&]() {
         dfree(lcol); dfree(llen); dfree(ucol); dfree(ulen); dfree(status); dfree(lrl);
-        dfree(url); dfree(lval); dfree(uval);
+        dfree(url); dfree(runs); dfree(lval); dfree(uval);
     };
     auto fail = [&](hec_status e) {
         cleanup();
@@ -371,6 +416,20 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
         P.n = n; P.p = p; P.tol = tol; P.rp = rowptr; P.ci = col; P.v = val;
         P.lcol = lcol; P.lval = lval; P.llen = llen; P.ucol = ucol; P.uval = uval; P.ulen = ulen;
         P.status = status;
+        // the runs (lrl and url hold the flags and their prefix until the row lengths take them)
+        const int gr = (n + 255) / 256;
+        k_run_flags<<<gr, 256, 0, s>>>(n, rowptr, col, lrl);
+        count_launch();
+        if ((st = exclusive_scan_i32(lrl, url, n, true, s))) return fail(st);
+        int nruns = 0;
+        if (cudaMemcpyAsync(&nruns, url + n, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess)
+            return fail(cuda_error(cudaGetLastError(), "ilut_factor: runs"));
+        if ((st = dalloc(&runs, (size_t)nruns + 1))) return fail(st);
+        k_run_starts<<<gr, 256, 0, s>>>(n, lrl, url, runs);
+        count_launch();
+        P.runs = runs;
+        P.nruns = nruns;
         P.budget = 4000000000LL;  // about two seconds of SM cycles per wait
         const void* k = (const void*)k_ilut;
         int h = 0, cap = 0;
@@ -388,6 +447,7 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
                           cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess))
                 return fail(cuda_error(cudaGetLastError(), "ilut_factor: memset"));
             P.cap = cap;
+            P.g = std::min(blocks * warps, std::max(kRunWarps, 2 * blocks * warps / std::max(1, nruns)));
             void* args[] = {&P};
             if (cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(warps * 32), args, smem, s) != cudaSuccess)
                 return fail(cuda_error(cudaGetLastError(), "ilut_factor: launch"));
