@@ -21,6 +21,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -68,26 +69,6 @@ __device__ __forceinline__ uint4 apply_mask(uint4 v, uint4 m) {
     return v;
 }
 
-// Stage the 34 x 6 x 3 halo of tile (bx, by, bz) into shared memory (zero outside the grid or the
-// sample), masked by `mask` when given.
-__device__ __forceinline__ void load_halo(const Geom& g, const __nv_bfloat16* __restrict__ X,
-                                          const __nv_bfloat16* __restrict__ mask, int bx, int by, int bz,
-                                          __nv_bfloat16 (*sx)[HY][HX][C]) {
-    const int sample = bz / g.zs, zl = bz - sample * g.zs;
-    for (int i = threadIdx.x; i < HZ * HY * HX * 2; i += blockDim.x) {
-        const int v = i >> 1, half = i & 1;
-        const int hx = v % HX, hy = (v / HX) % HY, hz = v / (HX * HY);
-        const int x = bx + hx - 1, y = by + hy - 1, z = zl + hz - 1;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (x >= 0 && x < g.nx && y >= 0 && y < g.ny && z >= 0 && z < g.zs) {
-            const long gi = (((long)sample * g.zs + z) * g.ny + y) * g.nx + x;
-            val = __ldg((const uint4*)X + gi * 2 + half);
-            if (mask) val = apply_mask(val, __ldg((const uint4*)mask + gi * 2 + half));
-        }
-        ((uint4*)&sx[0][0][0][0])[v * 2 + half] = val;
-    }
-}
-
 // ---- forward / data-gradient convolution ----------------------------------------------------
 // A block computes a 32 (x) x 4 (y) x 4 (z) output tile with 4 warps, warp w owning the z-plane w
 // of the tile (32 x 4 voxels = 2 m-tiles x 4 rows).  The 34 x 6 x 6 input halo and the weight
@@ -109,6 +90,11 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void* src, int by
 }
 __device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], unsigned addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_x4_t(unsigned (&r)[4], unsigned addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
 }
@@ -690,91 +676,146 @@ __global__ void __launch_bounds__(tc_threads(EXP), 2)
     if (warp == MMA_WARP) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TC_COLS));
 }
 
-// Weight and bias gradients of one layer: partial[block][tap][ci][co] = sum over this tile's voxels
+// Weight and bias gradients of one layer: partial[block][tap][ci][co] = sum over this block's voxels
 // of Ain[v + off(tap)][ci] * dZ[v][co], partial[block][WSZ + co] = sum of dZ[v][co];
 // dZ = dA masked by the layer's ReLU (mask = its output) when mask is given.
-__global__ void __launch_bounds__(kConvThreads) k_conv_wgrad(Geom g, const __nv_bfloat16* __restrict__ Ain,
-                                                             const __nv_bfloat16* __restrict__ dA,
-                                                             const __nv_bfloat16* __restrict__ mask,
-                                                             float* __restrict__ partial) {
-    __shared__ __align__(16) __nv_bfloat16 sx[HZ][HY][HX][C];
-    __shared__ __align__(16) __nv_bfloat16 sd[TY][TX][C];
+//   A block takes the tiles blockIdx.x, + gridDim.x, ... (32 x 4 x 1 voxels with a 34 x 6 x 3 halo)
+// and keeps its sums in registers, so 27.7 KB of partial sums are written once per block
+// (kWgradBlocks an SM) instead of once per tile: at 8 x 32^3 voxels 17 MB a layer instead of 57 MB,
+// and as much less for the reduction to read.  Warp w owns the taps w, w + 4, ...; a tile's products
+// are summed by the tensor cores from zero and added to the running sums in FP32.  Both operands are
+// voxel-major in shared memory and are transposed by ldmatrix; the dZ fragments of a tile (8 steps of
+// 16 voxels) serve all of a warp's taps.  Rows are swizzled as in the forward kernel.
+//   8 x 32^3 voxels, a layer: 46 us with a block per tile, scalar fragment loads and 2,048 partials, 25 us
+// so (a pass of net_backward with 3 / 4 blocks an SM: 392 / 397 us; 688 us at 46 us a layer).
+constexpr int kWgradBlocks = 3;
+constexpr int kWTaps = (NTAP + 3) / 4;
+
+__global__ void __launch_bounds__(kConvThreads, kWgradBlocks)
+    k_conv_wgrad(Geom g, int xt, int yt, int tiles, const __nv_bfloat16* __restrict__ Ain,
+                 const __nv_bfloat16* __restrict__ dA, const __nv_bfloat16* __restrict__ mask, float* __restrict__ partial) {
+    constexpr int KS = TX * TY / 16;  // steps of 16 voxels
+    __shared__ __align__(128) unsigned char s_x[HZ * HY * HX * 32];
+    __shared__ __align__(128) unsigned char s_d[TY * TX * 32];
     __shared__ float sbias[kConvThreads / 32][C];
-    const int bx = blockIdx.x * TX, by = blockIdx.y * TY, bz = blockIdx.z;
-    load_halo(g, Ain, nullptr, bx, by, bz, sx);
-    for (int i = threadIdx.x; i < TY * TX * 2; i += blockDim.x) {
-        const int v = i >> 1, half = i & 1;
-        const int lx = v % TX, ly = v / TX;
-        const int x = bx + lx, y = by + ly;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (x < g.nx && y < g.ny) {
-            const long gi = ((long)bz * g.ny + y) * g.nx + x;
-            val = __ldg((const uint4*)dA + gi * 2 + half);
-            if (mask) val = apply_mask(val, __ldg((const uint4*)mask + gi * 2 + half));
-        }
-        ((uint4*)&sd[0][0][0])[v * 2 + half] = val;
-    }
-    __syncthreads();
+    const unsigned sx = (unsigned)__cvta_generic_to_shared(s_x), sd = (unsigned)__cvta_generic_to_shared(s_d);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int gq = lane >> 2, t = lane & 3;
-    const long pbase = (long)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * PSZ;
-    // taps w, w + 4, w + 8, ... for this warp
-    for (int tap = w; tap < NTAP; tap += 4) {
-        const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-        float acc[2][4];
+    const int lr = lane & 7, lm = lane >> 3;             // ldmatrix: row of matrix lm
+    const int a_vox = lr + (lm >> 1) * 8, a_half = lm & 1;  // A: voxels 0-7 / 8-15, input channels 0-7 / 8-15
+    const int b_vox = lr + (lm & 1) * 8, b_half = lm >> 1;  // B: voxels 0-7 / 8-15, output channels 0-7 / 8-15
+    float acc[kWTaps][2][4], bsum = 0.f;
+#pragma unroll
+    for (int i = 0; i < kWTaps; ++i)
 #pragma unroll
         for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < TX * TY / 16; ++ks) {
-            const int vy = (ks * 16) / TX, vx0 = (ks * 16) % TX;
-            // A[m = ci][k = voxel]: Ain at the shifted voxel
-            const __nv_bfloat16* srow = &sx[dz][vy + dy][0][0];
-            unsigned af[4];
-            af[0] = pack2(srow[(vx0 + 2 * t + dx) * C + gq], srow[(vx0 + 2 * t + 1 + dx) * C + gq]);
-            af[1] = pack2(srow[(vx0 + 2 * t + dx) * C + gq + 8], srow[(vx0 + 2 * t + 1 + dx) * C + gq + 8]);
-            af[2] = pack2(srow[(vx0 + 2 * t + 8 + dx) * C + gq], srow[(vx0 + 2 * t + 9 + dx) * C + gq]);
-            af[3] = pack2(srow[(vx0 + 2 * t + 8 + dx) * C + gq + 8], srow[(vx0 + 2 * t + 9 + dx) * C + gq + 8]);
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                const int co = nt * 8 + gq;
-                unsigned bfr[2];
-                bfr[0] = pack2(sd[vy][vx0 + 2 * t][co], sd[vy][vx0 + 2 * t + 1][co]);
-                bfr[1] = pack2(sd[vy][vx0 + 2 * t + 8][co], sd[vy][vx0 + 2 * t + 9][co]);
-                mma_bf16(acc[nt], af, bfr);
-            }
+            for (int c = 0; c < 4; ++c) acc[i][nt][c] = 0.f;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int bx = tile % xt * TX, by = tile / xt % yt * TY, bz = tile / xt / yt;
+        const int sample = bz / g.zs, zl = bz - sample * g.zs;
+        __syncthreads();  // the tile before has been read
+        for (int i = threadIdx.x; i < HZ * HY * HX * 2; i += kConvThreads) {
+            const int v = i >> 1, half = i & 1;
+            const int hx = v % HX, hy = (v / HX) % HY, hz = v / (HX * HY);
+            const int x = bx + hx - 1, y = by + hy - 1, z = zl + hz - 1;
+            const bool inb = x >= 0 && x < g.nx && y >= 0 && y < g.ny && z >= 0 && z < g.zs;
+            const long gi = inb ? (((long)sample * g.zs + z) * g.ny + y) * g.nx + x : 0;
+            cp_async16(sx + swz(v, half), Ain + gi * C + half * 8, inb ? 16 : 0);
         }
+        for (int i = threadIdx.x; i < TY * TX * 2; i += kConvThreads) {
+            const int v = i >> 1, half = i & 1;
+            const int x = bx + v % TX, y = by + v / TX;
+            uint4 val = make_uint4(0, 0, 0, 0);
+            if (x < g.nx && y < g.ny) {
+                const long gi = ((long)bz * g.ny + y) * g.nx + x;
+                val = __ldg((const uint4*)dA + gi * 2 + half);
+                if (mask) val = apply_mask(val, __ldg((const uint4*)mask + gi * 2 + half));
+            }
+            *(uint4*)(s_d + swz(v, half)) = val;
+        }
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        unsigned bf[KS][4];
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) ldsm_x4_t(bf[ks], sd + swz(ks * 16 + b_vox, b_half));
+#pragma unroll
+        for (int i = 0; i < kWTaps; ++i) {
+            const int tap = w + 4 * i;
+            if (tap >= NTAP) break;
+            const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
+            float sum[2][4];
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) sum[nt][c] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+                const int vy = ks * 16 / TX, vx = ks * 16 % TX;
+                unsigned af[4];
+                ldsm_x4_t(af, sx + swz((dz * HY + vy + dy) * HX + vx + dx + a_vox, a_half));
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    const unsigned b2[2] = {bf[ks][2 * nt], bf[ks][2 * nt + 1]};
+                    mma_bf16(sum[nt], af, b2);
+                }
+            }
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[i][nt][c] += sum[nt][c];
+        }
+        // bias gradient: warp w sums rows y = w of the tile
+        if (lane < C) {
+            float s = 0.f;
+            for (int x = 0; x < TX; ++x)
+                s += __bfloat162float(*(const __nv_bfloat16*)(s_d + swz(w * TX + x, lane >> 3) + (lane & 7) * 2));
+            bsum += s;
+        }
+    }
+    float* out = partial + (long)blockIdx.x * PSZ;
+#pragma unroll
+    for (int i = 0; i < kWTaps; ++i) {
+        const int tap = w + 4 * i;
+        if (tap >= NTAP) break;
 #pragma unroll
         for (int nt = 0; nt < 2; ++nt) {
-            const int co = nt * 8 + 2 * t;
-            partial[pbase + (long)tap * C * C + gq * C + co] = acc[nt][0];
-            partial[pbase + (long)tap * C * C + gq * C + co + 1] = acc[nt][1];
-            partial[pbase + (long)tap * C * C + (gq + 8) * C + co] = acc[nt][2];
-            partial[pbase + (long)tap * C * C + (gq + 8) * C + co + 1] = acc[nt][3];
+            float* o = out + tap * C * C + gq * C + nt * 8 + 2 * t;
+            *(float2*)o = make_float2(acc[i][nt][0], acc[i][nt][1]);
+            *(float2*)(o + 8 * C) = make_float2(acc[i][nt][2], acc[i][nt][3]);
         }
     }
-    // bias gradient: warp w sums rows y = w of the tile
-    if (lane < C) {
-        float s = 0.f;
-        for (int x = 0; x < TX; ++x) s += __bfloat162float(sd[w][x][lane]);
-        sbias[w][lane] = s;
-    }
+    if (lane < C) sbias[w][lane] = bsum;
     __syncthreads();
     if (threadIdx.x < C) {
         float s = 0.f;
         for (int i = 0; i < kConvThreads / 32; ++i) s += sbias[i][threadIdx.x];
-        partial[pbase + WSZ + threadIdx.x] = s;
+        out[WSZ + threadIdx.x] = s;
     }
 }
 
-// grad[j] = sum over blocks of partial[b][j], in block order
-__global__ void k_reduce_partials(int nblk, const float* __restrict__ partial, float* __restrict__ grad) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= PSZ) return;
+// grad[j] = sum over blocks of partial[b][j] in a fixed order: kRedRows rows of threads each add
+// every kRedRows-th block, and their sums are added in row order.  (One thread a parameter, 28 blocks in
+// all, was a serial chain of as many loads as there are blocks: 83 us for 2,048 blocks; 9.4 us now for 456.)
+constexpr int kRedCols = 32, kRedRows = 16;
+__global__ void __launch_bounds__(kRedCols * kRedRows) k_reduce_partials(int nblk, const float* __restrict__ partial,
+                                                                         float* __restrict__ grad) {
+    __shared__ float red[kRedRows][kRedCols];
+    const int c = threadIdx.x % kRedCols, r = threadIdx.x / kRedCols;
+    const int j = blockIdx.x * kRedCols + c;
     float s = 0.f;
-    for (int b = 0; b < nblk; ++b) s += partial[(long)b * PSZ + j];
-    grad[j] = s;
+    if (j < PSZ) {
+#pragma unroll 4
+        for (int b = r; b < nblk; b += kRedRows) s += __ldg(partial + (long)b * PSZ + j);
+    }
+    red[r][c] = s;
+    __syncthreads();
+    if (r == 0 && j < PSZ) {
+        float t = 0.f;
+#pragma unroll
+        for (int i = 0; i < kRedRows; ++i) t += red[i][c];
+        grad[j] = t;
+    }
 }
 
 // From FP32 master parameters P[tap][ci][co] (+ bias) to the BF16 forward layout Wf[tap][co][ci]
@@ -897,8 +938,9 @@ hec_status refresh_weights(hec_net* N, cudaStream_t s) {
     return HEC_OK;
 }
 
-// grid of the weight-gradient kernel (one 32 x 4 x 1 tile per block)
-dim3 conv_grid(const Geom& g) { return dim3((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, g.nz); }
+// the weight-gradient kernel's 32 x 4 x 1 tiles, and its blocks
+int wgrad_tiles(const Geom& g) { return (g.nx + TX - 1) / TX * ((g.ny + TY - 1) / TY) * g.nz; }
+int wgrad_blocks(const Geom& g) { return std::max(1, std::min(wgrad_tiles(g), kWgradBlocks * num_sms())); }
 
 hec_status check_geom(const Geom& g) {
     if (g.nx <= 0 || g.ny <= 0 || g.nz <= 0 || g.zs <= 0 || g.nz % g.zs != 0 || (g.ny + TY - 1) / TY > 65535 ||
@@ -1034,13 +1076,13 @@ hec_status forward(hec_net* N, const Geom& g, const ConvIn& in, const ConvOut& l
 
 // backward from dA[0] = dLoss/dOutput (16-channel, channel 0); gradients into N->G
 hec_status backward(hec_net* N, const Geom& g, cudaStream_t s) {
-    const dim3 grid = conv_grid(g);
-    const long nblk = (long)grid.x * grid.y * grid.z;
+    const int nblk = wgrad_blocks(g), xt = (g.nx + TX - 1) / TX, yt = (g.ny + TY - 1) / TY;
     int cur = 0;
     for (int l = NL - 1; l >= 0; --l) {
         const __nv_bfloat16* mask = l == NL - 1 ? nullptr : N->act[l + 1];  // ReLU of layer l
-        k_conv_wgrad<<<grid, kConvThreads, 0, s>>>(g, N->act[l], N->dA[cur], mask, N->partial);
-        k_reduce_partials<<<(PSZ + 255) / 256, 256, 0, s>>>((int)nblk, N->partial, N->G + (long)l * PSZ);
+        k_conv_wgrad<<<nblk, kConvThreads, 0, s>>>(g, xt, yt, wgrad_tiles(g), N->act[l], N->dA[cur], mask, N->partial);
+        k_reduce_partials<<<(PSZ + kRedCols - 1) / kRedCols, kRedCols * kRedRows, 0, s>>>(nblk, N->partial,
+                                                                                          N->G + (long)l * PSZ);
         count_launch(2);
         if (l > 0) {
             const ConvIn din{N->dA[cur], mask, nullptr, nullptr, nullptr};
@@ -1065,8 +1107,7 @@ hec_status net_apply_field(hec_net* N, int nx, int ny, int nz, const double* r, 
     Geom g{nx, ny, nz, nz};
     HEC_CHECK(check_geom(g));
     const long nvox = (long)nx * ny * nz;
-    const dim3 grid = conv_grid(g);
-    HEC_CHECK(ensure(N, nvox, (long)grid.x * grid.y * grid.z));
+    HEC_CHECK(ensure(N, nvox, wgrad_blocks(g)));
     return forward(N, g, ConvIn{nullptr, nullptr, r, sigma, aux}, ConvOut{nullptr, nullptr, 1.f, c, sigma}, s);
 }
 
@@ -1196,8 +1237,7 @@ HEC_API hec_status net_forward(hec_net* N, int nx, int ny, int nz, int zs, const
     HEC_CHECK(check_geom(g));
     cudaStream_t s = S(stream);
     const long nvox = (long)nx * ny * nz;
-    const dim3 grid = conv_grid(g);
-    HEC_CHECK(ensure(N, nvox, (long)grid.x * grid.y * grid.z));
+    HEC_CHECK(ensure(N, nvox, wgrad_blocks(g)));
     HEC_CUDA(cudaMemcpyAsync(N->act[0], x_in, sizeof(__nv_bfloat16) * C * nvox, cudaMemcpyDeviceToDevice, s));
     HEC_CHECK(forward(N, g, ConvIn{N->act[0], nullptr, nullptr, nullptr, nullptr},
                       ConvOut{N->act[NL], N->out, 1.f, nullptr, nullptr}, s));
@@ -1216,8 +1256,7 @@ static hec_status net_backward_impl(hec_net* N, int nx, int ny, int nz, int zs, 
     Geom g{nx, ny, nz, zs};
     HEC_CHECK(check_geom(g));
     const long nvox = (long)nx * ny * nz;
-    const dim3 grid = conv_grid(g);
-    HEC_CHECK(ensure(N, nvox, (long)grid.x * grid.y * grid.z));
+    HEC_CHECK(ensure(N, nvox, wgrad_blocks(g)));
     HEC_CUDA(cudaMemcpyAsync(N->act[0], x_in, sizeof(__nv_bfloat16) * C * nvox, cudaMemcpyDeviceToDevice, s));
     HEC_CHECK(forward(N, g, ConvIn{N->act[0], nullptr, nullptr, nullptr, nullptr},
                       ConvOut{N->act[NL], N->out, 1.f, nullptr, nullptr}, s));
