@@ -6,8 +6,8 @@
 // out statically, chunk c to warp c mod W, under a cooperative launch that guarantees all warps
 // are resident, so the warp holding the earliest unfinished chunk can always proceed.
 //
-// The map is a stable counting sort of rows by level (least-significant-digit radix passes of
-// 8 bits over the level), which keeps the rows of each level in ascending order of the lower
+// The map is a stable counting sort of rows by level (least-significant-digit radix passes
+// over the level), which keeps the rows of each level in ascending order of the lower
 // problem's index as Eq. 3 requires; it is exact integer work and bit-identical to the plain
 // serial construction.
 #include <algorithm>
@@ -169,78 +169,108 @@ __global__ void __launch_bounds__(256, 8) k_levels(int n, const int* __restrict_
 }
 
 // ---- stable counting sort by level ------------------------------------------------------------
-constexpr int kRadixBits = 8;
-constexpr int kDigits = 1 << kRadixBits;
+// Least-significant-digit passes of at most kRadixBits bits, as few and as even as the largest key
+// allows: up to 1024 levels are one pass.  A tile of kTileItems keys is one warp's; what a pass
+// costs besides the keys is its table of (digits x tiles) counts and their scan.
+constexpr int kRadixBits = 10;
 constexpr int kTileItems = 32 * 32;  // keys per warp tile
-constexpr int kSortWarps = 8;        // warps per block
+constexpr int kSortWarps = 4;        // warps per block (4 x 1024 counters: 16 KB of shared memory)
 
-// keys for the first pass: key[t] = level of the row at position t of the lower problem,
-// val[t] = that original row
-__global__ void k_init_keys(int n, int uplo, const int* __restrict__ level, int* key, int* val) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    int i = uplo ? n - 1 - t : t;
-    key[t] = level[i];
-    val[t] = i;
-}
+// key and value at position t: from the arrays, or, in the first pass of the level sort, the level of
+// the row at position t of the lower problem and that original row
+struct SortIn {
+    const int* key;
+    const int* val;
+    const int* level;  // not NULL: the first pass of the level sort
+    int uplo;
+    __device__ __forceinline__ int row(int n, long t) const { return uplo ? n - 1 - (int)t : (int)t; }
+    __device__ __forceinline__ int k(int n, long t) const { return level ? level[row(n, t)] : key[t]; }
+    __device__ __forceinline__ int v(int n, long t) const { return level ? row(n, t) : val[t]; }
+};
 
-__global__ void k_digit_count(int n, const int* __restrict__ key, int shift, int ntiles, int* counts) {
-    __shared__ int cnt[kSortWarps][kDigits];
+__global__ void k_digit_count(int n, SortIn in, int shift, int bits, int ntiles, int* counts) {
+    extern __shared__ int sort_smem[];
+    const int digits = 1 << bits;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int* cnt = sort_smem + warp * digits;
     const int tile = blockIdx.x * kSortWarps + warp;
-    for (int d = lane; d < kDigits; d += 32) cnt[warp][d] = 0;
+    for (int d = lane; d < digits; d += 32) cnt[d] = 0;
     __syncwarp();
     if (tile < ntiles) {
-        long base = (long)tile * kTileItems;
+        const long base = (long)tile * kTileItems;
+#pragma unroll 8
         for (int k = lane; k < kTileItems; k += 32) {
-            long t = base + k;
-            if (t < n) atomicAdd(&cnt[warp][(key[t] >> shift) & (kDigits - 1)], 1);
+            const long t = base + k;
+            if (t < n) atomicAdd(cnt + ((in.k(n, t) >> shift) & (digits - 1)), 1);
         }
         __syncwarp();
-        for (int d = lane; d < kDigits; d += 32) counts[(long)d * ntiles + tile] = cnt[warp][d];
+        for (int d = lane; d < digits; d += 32) counts[(long)d * ntiles + tile] = cnt[d];
     }
 }
 
-__global__ void k_digit_scatter(int n, const int* __restrict__ key, const int* __restrict__ val, int shift, int ntiles,
-                                const int* __restrict__ offs, int* okey, int* oval) {
-    __shared__ int base[kSortWarps][kDigits];
+// okey / oval: the sorted pairs (okey may be NULL); inv (may be NULL): inv[value] = its position
+__global__ void k_digit_scatter(int n, SortIn in, int shift, int bits, int ntiles, const int* __restrict__ offs, int* okey,
+                                int* oval, int* inv) {
+    extern __shared__ int sort_smem[];
+    const int digits = 1 << bits;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int* base = sort_smem + warp * digits;
     const int tile = blockIdx.x * kSortWarps + warp;
     if (tile >= ntiles) return;  // whole warp leaves together
-    for (int d = lane; d < kDigits; d += 32) base[warp][d] = offs[(long)d * ntiles + tile];
+    for (int d = lane; d < digits; d += 32) base[d] = offs[(long)d * ntiles + tile];
     __syncwarp();
     const unsigned lt = (1u << lane) - 1u;
-    long t0 = (long)tile * kTileItems;
-    for (int r = 0; r < kTileItems; r += 32) {
-        long t = t0 + r + lane;
-        bool ok = t < n;
-        int k = ok ? key[t] : 0;
-        int d = ok ? ((k >> shift) & (kDigits - 1)) : kDigits + lane;  // invalid lanes get unique digits
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        int rank = __popc(peers & lt);
-        int pos = ok ? base[warp][d] + rank : 0;
+    const long t0 = (long)tile * kTileItems;
+    long t = t0 + lane;
+    int kn = t < n ? in.k(n, t) : 0;  // one step ahead: its load overlaps the ranking
+    for (int r = 0; r < kTileItems && t0 + r < n; r += 32, t += 32) {
+        const bool ok = t < n;
+        const int k = kn;
+        if (t + 32 < n) kn = in.k(n, t + 32);
+        const int d = ok ? ((k >> shift) & (digits - 1)) : digits + lane;  // invalid lanes get unique digits
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const int rank = __popc(peers & lt);
+        const int pos = ok ? base[d] + rank : 0;
         __syncwarp();
-        if (ok && rank == 0) base[warp][d] += __popc(peers);
+        if (ok && rank == 0) base[d] += __popc(peers);
         __syncwarp();
         if (ok) {
-            okey[pos] = k;
-            oval[pos] = val[t];
+            const int v = in.v(n, t);
+            if (okey) okey[pos] = k;
+            oval[pos] = v;
+            if (inv) inv[v] = pos;
         }
     }
 }
 
-__global__ void k_perm_from_order(int n, const int* __restrict__ order, int* perm, int* iperm) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    int i = order[p];
-    iperm[p] = i;
-    perm[i] = p;
+// level_ptr from the scanned counts of a single pass (the first position of each digit), or from the
+// sorted keys (every level has a row)
+__global__ void k_level_ptr_offs(int nlev, int n, int ntiles, const int* __restrict__ offs, int* level_ptr) {
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l < nlev) level_ptr[l] = offs[(long)l * ntiles];
+    if (l == nlev) level_ptr[l] = n;
+}
+__global__ void k_level_ptr_keys(int nlev, int n, const int* __restrict__ key, int* level_ptr) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < n && (p == 0 || key[p] != key[p - 1])) level_ptr[key[p]] = p;
+    if (p == 0) level_ptr[nlev] = n;
 }
 
-__global__ void k_level_hist(int n, const int* __restrict__ level, int* hist) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) atomicAdd(hist + level[i], 1);
-}
+// One sort by keys in [0, max_key]: passes and bits a pass
+struct SortShape {
+    int passes, bits, ntiles, blocks;
+    size_t smem;
+    SortShape(int n, long long max_key) {
+        int b = 0;
+        while ((1LL << b) <= max_key) b++;
+        passes = std::max(1, (b + kRadixBits - 1) / kRadixBits);
+        bits = std::max(1, (b + passes - 1) / passes);
+        ntiles = (n + kTileItems - 1) / kTileItems;
+        blocks = (ntiles + kSortWarps - 1) / kSortWarps;
+        smem = sizeof(int) * ((size_t)kSortWarps << bits);
+    }
+    size_t counts() const { return ((size_t)ntiles << bits) + 1; }
+};
 
 }  // namespace
 
@@ -305,39 +335,34 @@ hec_status compute_levels(int n, const int* rp, const int* col, int dep_side, he
         HEC_CUDA(cudaStreamSynchronize(s));
         return HEC_OK;
     }
-    // level_ptr: histogram + exclusive scan
-    HEC_CUDA(cudaMemsetAsync(lv->level_ptr, 0, sizeof(int) * ((size_t)lv->nlev + 1), s));
-    k_level_hist<<<(n + 255) / 256, 256, 0, s>>>(n, lv->level, lv->level_ptr);
-    HEC_LAUNCHED();
-    HEC_CHECK(exclusive_scan_i32(lv->level_ptr, lv->level_ptr, lv->nlev, true, s));
-    // stable LSD radix sort of (level, position) pairs
+    // stable LSD radix sort of (level, row): the last pass writes the map and its inverse
+    const SortShape sh(n, lv->nlev - 1);
     int *k0 = nullptr, *v0 = nullptr, *k1 = nullptr, *v1 = nullptr, *counts = nullptr;
-    int ntiles = (n + kTileItems - 1) / kTileItems;
     hec_status st = HEC_OK;
-    if ((st = dalloc(&k0, (size_t)n)) || (st = dalloc(&v0, (size_t)n)) || (st = dalloc(&k1, (size_t)n)) ||
-        (st = dalloc(&v1, (size_t)n)) || (st = dalloc(&counts, (size_t)kDigits * ntiles + 1))) {
+    if ((st = dalloc(&counts, sh.counts())) ||
+        (sh.passes > 1 && ((st = dalloc(&k0, (size_t)n)) || (st = dalloc(&v0, (size_t)n)) || (st = dalloc(&k1, (size_t)n)) ||
+                           (st = dalloc(&v1, (size_t)n))))) {
         dfree(k0); dfree(v0); dfree(k1); dfree(v1); dfree(counts);
         return st;
     }
-    k_init_keys<<<(n + 255) / 256, 256, 0, s>>>(n, dep_side, lv->level, k0, v0);
-    count_launch();
-    int bits = 0;
-    while ((1LL << bits) < (long long)lv->nlev) bits++;
-    int passes = std::max(1, (bits + kRadixBits - 1) / kRadixBits);
-    int sblocks = (ntiles + kSortWarps - 1) / kSortWarps;
-    for (int ps = 0; ps < passes && st == HEC_OK; ++ps) {
-        int shift = ps * kRadixBits;
-        k_digit_count<<<sblocks, 32 * kSortWarps, 0, s>>>(n, k0, shift, ntiles, counts);
+    for (int ps = 0; ps < sh.passes && st == HEC_OK; ++ps) {
+        const SortIn in{k0, v0, ps == 0 ? lv->level : nullptr, dep_side};
+        const bool last = ps == sh.passes - 1;
+        k_digit_count<<<sh.blocks, 32 * kSortWarps, sh.smem, s>>>(n, in, ps * sh.bits, sh.bits, sh.ntiles, counts);
         count_launch();
-        st = exclusive_scan_i32(counts, counts, kDigits * ntiles, false, s);
+        st = exclusive_scan_i32(counts, counts, (int)(sh.counts() - 1), false, s);
         if (st != HEC_OK) break;
-        k_digit_scatter<<<sblocks, 32 * kSortWarps, 0, s>>>(n, k0, v0, shift, ntiles, counts, k1, v1);
+        k_digit_scatter<<<sh.blocks, 32 * kSortWarps, sh.smem, s>>>(n, in, ps * sh.bits, sh.bits, sh.ntiles, counts, k1,
+                                                                    last ? lv->iperm : v1, last ? lv->perm : nullptr);
         count_launch();
         std::swap(k0, k1);
         std::swap(v0, v1);
     }
     if (st == HEC_OK) {
-        k_perm_from_order<<<(n + 255) / 256, 256, 0, s>>>(n, v0, lv->perm, lv->iperm);
+        if (sh.passes == 1)
+            k_level_ptr_offs<<<lv->nlev / 256 + 1, 256, 0, s>>>(lv->nlev, n, sh.ntiles, counts, lv->level_ptr);
+        else
+            k_level_ptr_keys<<<(n + 255) / 256, 256, 0, s>>>(lv->nlev, n, k0, lv->level_ptr);
         count_launch();
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -347,29 +372,25 @@ hec_status compute_levels(int n, const int* rp, const int* col, int dep_side, he
     return st;
 }
 
-// Stable sort of (key, val) pairs by key, 0 <= key <= max_key, in place (LSD radix, 8-bit
-// digits).  Synchronizes.
+// Stable sort of (key, val) pairs by key, 0 <= key <= max_key, in place (LSD radix).  Synchronizes.
 hec_status sort_pairs_i32(int* keys, int* vals, int n, int max_key, cudaStream_t s) {
     if (n <= 1) return HEC_OK;
     int *k1 = nullptr, *v1 = nullptr, *counts = nullptr;
-    const int ntiles = (n + kTileItems - 1) / kTileItems;
+    const SortShape sh(n, max_key);
     hec_status st = HEC_OK;
-    if ((st = dalloc(&k1, (size_t)n)) || (st = dalloc(&v1, (size_t)n)) ||
-        (st = dalloc(&counts, (size_t)kDigits * ntiles + 1))) {
+    if ((st = dalloc(&k1, (size_t)n)) || (st = dalloc(&v1, (size_t)n)) || (st = dalloc(&counts, sh.counts()))) {
         dfree(k1); dfree(v1); dfree(counts);
         return st;
     }
-    int bits = 0;
-    while ((1LL << bits) <= (long long)max_key) bits++;
-    const int passes = std::max(1, (bits + kRadixBits - 1) / kRadixBits);
-    const int sblocks = (ntiles + kSortWarps - 1) / kSortWarps;
     int *ka = keys, *va = vals, *kb = k1, *vb = v1;
-    for (int ps = 0; ps < passes && st == HEC_OK; ++ps) {
-        k_digit_count<<<sblocks, 32 * kSortWarps, 0, s>>>(n, ka, ps * kRadixBits, ntiles, counts);
+    for (int ps = 0; ps < sh.passes && st == HEC_OK; ++ps) {
+        const SortIn in{ka, va, nullptr, 0};
+        k_digit_count<<<sh.blocks, 32 * kSortWarps, sh.smem, s>>>(n, in, ps * sh.bits, sh.bits, sh.ntiles, counts);
         count_launch();
-        st = exclusive_scan_i32(counts, counts, kDigits * ntiles, false, s);
+        st = exclusive_scan_i32(counts, counts, (int)(sh.counts() - 1), false, s);
         if (st != HEC_OK) break;
-        k_digit_scatter<<<sblocks, 32 * kSortWarps, 0, s>>>(n, ka, va, ps * kRadixBits, ntiles, counts, kb, vb);
+        k_digit_scatter<<<sh.blocks, 32 * kSortWarps, sh.smem, s>>>(n, in, ps * sh.bits, sh.bits, sh.ntiles, counts, kb, vb,
+                                                                    nullptr);
         count_launch();
         std::swap(ka, kb);
         std::swap(va, vb);

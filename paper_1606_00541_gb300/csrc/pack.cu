@@ -36,40 +36,42 @@ template <> __device__ __forceinline__ double widen<double>(double v) { return v
 template <> __device__ __forceinline__ double widen<float>(float v) { return (double)v; }
 template <> __device__ __forceinline__ double widen<__nv_bfloat16>(__nv_bfloat16 v) { return (double)__bfloat162float(v); }
 
-// eligible entries per new row (off-diagonals in triangular mode)
-__global__ void k_row_counts(int n, const int* __restrict__ rp, const int* __restrict__ iperm, int tri, int* cnt,
-                             int* maxcnt) {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
-    int c = 0;
-    if (r < n) {
-        int i = tri ? iperm[r] : r;
-        c = rp[i + 1] - rp[i] - (tri ? 1 : 0);
-        cnt[r] = c;
-    }
-    for (int o = 16; o; o >>= 1) c = max(c, __shfl_xor_sync(0xffffffffu, c, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(maxcnt, c);
-}
-
-// histogram of the row counts: few distinct values, so each block counts the small ones in shared
-// memory and adds its totals once (a global atomic per row would serialise on a handful of bins)
-__global__ void k_count_hist(int n, const int* __restrict__ cnt, int nbins, int* hist) {
+// Histogram of the rows' eligible entries (off-diagonals in triangular mode; rows in any order), counts
+// of nbins - 1 and more in the last bin, and the largest count in *maxcnt.  Few distinct values: each
+// block counts the small ones in shared memory and adds its totals once (a global atomic per row or per
+// warp would serialise on a handful of words).
+__global__ void k_count_hist(int n, const int* __restrict__ rp, int tri, int nbins, int* hist, int* maxcnt) {
     __shared__ int sh[64];
     for (int t = threadIdx.x; t < 64; t += blockDim.x) sh[t] = 0;
     __syncthreads();
+    int most = 0;
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-        const int c = cnt[r];
-        if (c < 64) atomicAdd(sh + c, 1);
-        else atomicAdd(hist + c, 1);
+        const int c = rp[r + 1] - rp[r] - (tri ? 1 : 0);
+        most = max(most, c);
+        const int bin = min(c, nbins - 1);
+        if (bin < 64) atomicAdd(sh + bin, 1);
+        else atomicAdd(hist + bin, 1);
     }
     __syncthreads();
     for (int t = threadIdx.x; t < 64 && t < nbins; t += blockDim.x)
         if (sh[t]) atomicAdd(hist + t, sh[t]);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((threadIdx.x & 31) == 0 && most > *(volatile int*)maxcnt) atomicMax(maxcnt, most);
 }
 
-__global__ void k_tail_len(int n, const int* __restrict__ cnt, int w, int tri, int* tlen) {
+__global__ void k_tail_len(int n, const int* __restrict__ rp, const int* __restrict__ iperm, int w, int tri, int* tlen) {
     int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) tlen[r] = max(0, cnt[r] - w) + (tri ? 1 : 0);
+    if (r >= n) return;
+    const int i = tri ? iperm[r] : r;
+    tlen[r] = max(0, rp[i + 1] - rp[i] - (tri ? 1 : 0) - w) + (tri ? 1 : 0);
 }
+
+// One thread per new row.  A factor's row of at most kPackRegs entries (the stencil factors) is held
+// in registers: each column is read and mapped once, the ranks come from register compares, and the
+// slab slots are written in slot order, so a warp's stores of a slot are one segment.  Longer rows read
+// their columns again for every rank.  FP32 packing of a 7-point 128^3 factor, reading again / from
+// registers: 152 / 70 us (a general matrix, whose ranks are its CSR order, needs neither: 55 / 60 us).
+constexpr int kPackRegs = 8;
 
 template <typename VT>
 __global__ void k_pack(int n, int ld, int w, int tri, const int* __restrict__ rp, const int* __restrict__ col,
@@ -87,6 +89,61 @@ __global__ void k_pack(int n, int ld, int w, int tri, const int* __restrict__ rp
     int i = tri ? iperm[r] : r;
     int a = rp[i], b = rp[i + 1];
     int t0 = tptr[r];
+    if (tri && b - a <= kPackRegs) {
+        int nc[kPackRegs], rank[kPackRegs];
+        double v[kPackRegs], d = 0.0;
+#pragma unroll
+        for (int e = 0; e < kPackRegs; ++e) {
+            nc[e] = a + e < b ? __ldg(col + a + e) : -1;
+            v[e] = a + e < b ? __ldg(val + a + e) : 0.0;
+        }
+#pragma unroll
+        for (int e = 0; e < kPackRegs; ++e) {
+            if (nc[e] == i) {
+                d = v[e];
+                nc[e] = -1;
+            } else if (nc[e] >= 0) {
+                nc[e] = __ldg(perm + nc[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < kPackRegs; ++e) {
+            rank[e] = -1;
+            if (nc[e] >= 0) {
+                rank[e] = 0;
+#pragma unroll
+                for (int f = 0; f < kPackRegs; ++f) rank[e] += nc[f] >= 0 && nc[f] < nc[e];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kPackRegs; ++k) {
+            if (k >= w) break;
+            int c = -1;
+            double x = 0.0;
+#pragma unroll
+            for (int e = 0; e < kPackRegs; ++e)
+                if (rank[e] == k) {
+                    c = nc[e];
+                    x = v[e];
+                }
+            ell_col[(long)k * ld + r] = c;
+            ell_val[(long)k * ld + r] = cvt<VT>(x);
+        }
+        for (int k = kPackRegs; k < w; ++k) {
+            ell_col[(long)k * ld + r] = -1;
+            ell_val[(long)k * ld + r] = cvt<VT>(0.0);
+        }
+#pragma unroll
+        for (int e = 0; e < kPackRegs; ++e)
+            if (rank[e] >= w) {
+                tcol[t0 + rank[e] - w] = nc[e];
+                tval[t0 + rank[e] - w] = cvt<VT>(v[e]);
+            }
+        const int te = tptr[r + 1] - 1;
+        tcol[te] = r;
+        tval[te] = cvt<VT>(d);
+        return;
+    }
     int cnt = 0;
     for (int p = a; p < b; ++p) {
         int j = col[p];
@@ -226,54 +283,51 @@ HEC_API hec_status hec_from_csr(int n, const int* rowptr, const int* col, const 
     M->vdt = vdt;
     M->lv = lv;
     int* cnt = nullptr;
-    int* small = nullptr;  // [0] max count, [1] tail total
+    int* hist = nullptr;
     hec_status st = HEC_OK;
     auto fail = [&](hec_status e) {
         dfree(cnt);
-        dfree(small);
+        dfree(hist);
         free_matrix(M);
         return e;
     };
-    if ((st = dalloc(&cnt, (size_t)n + 1)) || (st = dalloc(&small, 2))) return fail(st);
+    if ((st = dalloc(&cnt, (size_t)n + 1))) return fail(st);
     if ((st = dalloc(&M->tptr, (size_t)n + 1))) return fail(st);
-    cudaMemsetAsync(small, 0, 2 * sizeof(int), s);
     const int* iperm = tri ? lv->iperm : nullptr;
     const int* perm = tri ? lv->perm : nullptr;
     int g = (n + 255) / 256;
-    if (n > 0) {
-        k_row_counts<<<g, 256, 0, s>>>(n, rowptr, iperm, tri, cnt, small);
-        count_launch();
-    }
     int w = ell_width;
     if (w < 0) {
-        int maxcnt = 0;
-        if (cudaMemcpyAsync(&maxcnt, small, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            return fail(cuda_error(cudaGetLastError(), "hec_from_csr: count"));
-        int* hist = nullptr;
-        if ((st = dalloc(&hist, (size_t)maxcnt + 1))) return fail(st);
-        cudaMemsetAsync(hist, 0, sizeof(int) * ((size_t)maxcnt + 1), s);
-        if (n > 0) {
-            k_count_hist<<<std::min(g, 4 * num_sms()), 256, 0, s>>>(n, cnt, maxcnt + 1, hist);
-            count_launch();
+        // row counts up to 1023 in one pass; a matrix with longer rows is counted again with every bin
+        std::vector<int> h;
+        for (int nbins = 1024;;) {
+            if ((st = dalloc(&hist, (size_t)nbins + 1))) return fail(st);
+            cudaMemsetAsync(hist, 0, sizeof(int) * ((size_t)nbins + 1), s);
+            if (n > 0) {
+                k_count_hist<<<std::min(g, 4 * num_sms()), 256, 0, s>>>(n, rowptr, tri, nbins, hist, hist + nbins);
+                count_launch();
+            }
+            h.resize((size_t)nbins + 1);
+            cudaError_t e = cudaMemcpyAsync(h.data(), hist, sizeof(int) * h.size(), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) return fail(cuda_error(e, "hec_from_csr: histogram"));
+            dfree(hist);
+            hist = nullptr;
+            if (h[nbins] < nbins) break;
+            nbins = h[nbins] + 1;
         }
-        std::vector<int> h((size_t)maxcnt + 1);
-        cudaError_t e = cudaMemcpyAsync(h.data(), hist, sizeof(int) * h.size(), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        dfree(hist);
-        if (e != cudaSuccess) return fail(cuda_error(e, "hec_from_csr: histogram"));
         // largest w with #rows(count >= w) >= ceil(0.65 n)
         long long need = (long long)((65LL * n + 99) / 100);
         long long atleast = 0;
         w = 0;
-        for (int c = maxcnt; c >= 1; --c) {
+        for (int c = (int)h.size() - 2; c >= 1; --c) {
             atleast += h[c];
             if (n > 0 && atleast >= need) { w = c; break; }
         }
     }
     M->w = w;
     if (n > 0) {
-        k_tail_len<<<g, 256, 0, s>>>(n, cnt, w, tri, cnt);
+        k_tail_len<<<g, 256, 0, s>>>(n, rowptr, iperm, w, tri, cnt);
         count_launch();
     }
     if ((st = exclusive_scan_i32(cnt, M->tptr, n, true, s))) return fail(st);
@@ -293,7 +347,6 @@ HEC_API hec_status hec_from_csr(int n, const int* rowptr, const int* col, const 
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(cuda_error(e, "hec_from_csr: pack"));
     dfree(cnt);
-    dfree(small);
     *out = M;
     return HEC_OK;
 }

@@ -1431,6 +1431,55 @@ __global__ void k_repack(int n, int ld, int w, const int* __restrict__ rowg, con
     auto col_of = [&](int e) { return sigma[e < nell ? ec[(long)e * ld + g] : tc[t0 + e - nell]]; };
     auto val_of = [&](int e) { return e < nell ? ev[(long)e * ld + g] : tv[t0 + e - nell]; };
     const int nt0 = ntp[r];
+    constexpr int kRegs = 8;
+    if (cnt <= kRegs && w <= kRegs) {  // as in the packing kernel: short rows from registers, slots in order
+        int c[kRegs], rank[kRegs];
+        VT v[kRegs];
+#pragma unroll
+        for (int e = 0; e < kRegs; ++e) {
+            c[e] = -1;
+            v[e] = (VT)0.0f;
+            if (e < cnt) {
+                c[e] = e < nell ? ec[(long)e * ld + g] : tc[t0 + e - nell];
+                v[e] = val_of(e);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < kRegs; ++e)
+            if (c[e] >= 0) c[e] = sigma[c[e]];
+#pragma unroll
+        for (int e = 0; e < kRegs; ++e) {
+            rank[e] = -1;
+            if (c[e] >= 0) {
+                rank[e] = 0;
+#pragma unroll
+                for (int f = 0; f < kRegs; ++f) rank[e] += c[f] >= 0 && c[f] < c[e];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kRegs; ++k) {
+            if (k >= w) break;
+            int cc = -1;
+            VT vv = (VT)0.0f;
+#pragma unroll
+            for (int e = 0; e < kRegs; ++e)
+                if (rank[e] == k) {
+                    cc = c[e];
+                    vv = v[e];
+                }
+            nec[(long)k * ld + r] = cc;
+            nev[(long)k * ld + r] = vv;
+        }
+#pragma unroll
+        for (int e = 0; e < kRegs; ++e)
+            if (rank[e] >= w) {
+                ntc[nt0 + rank[e] - w] = c[e];
+                ntv[nt0 + rank[e] - w] = v[e];
+            }
+        ntc[ntp[r + 1] - 1] = r;
+        ntv[ntp[r + 1] - 1] = tv[tp[g + 1] - 1];
+        return;
+    }
     for (int e = 0; e < cnt; ++e) {
         const int c = col_of(e);
         int rank = 0;
