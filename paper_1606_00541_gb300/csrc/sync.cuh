@@ -28,6 +28,17 @@ __device__ __forceinline__ unsigned int ld_relaxed_u32(const void* p) {
     asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
+// The same loads under a predicate, `v` kept where it is false.  Predicated in the instruction, so a poll
+// of several words issues all of its loads before the first is looked at: with a branch and a test
+// around each, the words of a poll arrive one L2 round trip after the other.
+__device__ __forceinline__ void ld_relaxed_if(bool on, const void* p, unsigned long long& v) {
+    asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\n@q ld.relaxed.gpu.global.b64 %0, [%1];\n}"
+                 : "+l"(v) : "l"(p), "r"((unsigned)on));
+}
+__device__ __forceinline__ void ld_relaxed_if(bool on, const void* p, unsigned int& v) {
+    asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\n@q ld.relaxed.gpu.global.b32 %0, [%1];\n}"
+                 : "+r"(v) : "l"(p), "r"((unsigned)on));
+}
 __device__ __forceinline__ void st_relaxed_u64(void* p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
