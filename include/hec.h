@@ -193,7 +193,11 @@ typedef struct {
 
 /* A solve plan for one triangular factor: its HEC form and level analysis (both borrowed; they
  * must outlive the plan) plus the workspace for up to max_nrhs right-hand sides
- * (1 <= max_nrhs <= 16).  tune may be NULL for defaults. */
+ * (1 <= max_nrhs <= 16).  tune may be NULL for defaults.
+ * A plan for one right-hand side with the default launch shape and lanes per row also gets, where it
+ * pays and device memory allows, the range schedule: contiguous ranges of original rows, one resident
+ * block each with its solution in shared memory, results as the global schedule's bit for bit.  It
+ * keeps a copy of the factor's column indices and two n-entry solution buffers. */
 hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* lv, int max_nrhs,
                               const hec_tune* tune, sptrsv_plan** out);
 hec_status sptrsv_plan_destroy(sptrsv_plan* p);
@@ -238,7 +242,8 @@ int sptrsv_partition_capacity(const sptrsv_plan* p, int threads);
  * fastest of the candidates in the plan; `out` (host, may be NULL) receives the choice.
  * Candidates: launch shapes block_threads in {128, 256} x blocks_per_sm in {2, 4, 8, 16} (those
  * that fit 2048 threads per SM); for nrhs = 1 also lanes per row in {1, 2, 4, 8} (one thread per
- * row against several lanes sharing a long row), and, when the plan has a partition
+ * row against several lanes sharing a long row), the plan's range schedule when it has one
+ * (sptrsv_plan_create), and, when the plan has a partition
  * (sptrsv_plan_partition), the partitioned schedule against the best global one (a plan whose
  * global schedule wins keeps its partition unused; partitioning it again re-enables it).
  * Results are cached per (rows, slab width, tail entries, levels, value type, nrhs rounded up to
@@ -253,8 +258,8 @@ hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void* stream
  * from 0 to n); the HEC factor (tail row pointers increasing from 0 to tail_nnz, slab columns in
  * [-1, n) with padding only after a row's entries, tail off-diagonals only after a full slab,
  * every off-diagonal in an earlier level than its row, the diagonal last in the tail and
- * nonzero); every chunk table (in order, each chunk inside one level, covering [0, n)); and, for a
- * partitioned plan, the row map (a permutation), the part tables, the repacked factor and the
+ * nonzero); every chunk table (in order, each chunk inside one level, covering [0, n)); the range
+ * schedule's chunks and coded columns; and, for a partitioned plan, the row map (a permutation), the part tables, the repacked factor and the
  * part chunks.  Returns HEC_OK, or HEC_ERR_OUT_OF_BOUNDS with hec_last_error() naming the first
  * failing check and index.  Reads only the plan; synchronizes `stream`. */
 hec_status sptrsv_plan_check(const sptrsv_plan* p, void* stream);

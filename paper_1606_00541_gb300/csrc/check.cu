@@ -16,6 +16,8 @@
 //   4. a partition, when set: rowg a permutation of [0, n), part_row non-decreasing from 0 to n,
 //      each part's chunks inside the part, level-aligned and covering it, and the repacked factor
 //      with columns in [-1, n) whose dependencies lie in earlier levels of the level order.
+//   5. the range schedule, when the plan has it: every row in exactly one chunk, of its range and of one
+//      level, each range's chunks in level order, and the coded columns those of the factor.
 // The first failure found (the lowest check number, then the lowest row) is reported as
 // HEC_ERR_OUT_OF_BOUNDS with a message naming the check and the row.  The plan is not changed.
 #include <algorithm>
@@ -133,9 +135,54 @@ __global__ void k_check_part_chunks(int nparts, const int* __restrict__ part_row
     }
 }
 
+// the range schedule: every row in exactly one chunk (`seen`), of its range and of one level, a range's
+// chunks in level order; the columns those of the factor in original numbering
+__global__ void k_check_range_chunks(int n, int nparts, int rows, const int* __restrict__ part_chunk,
+                                     const int2* __restrict__ ch, int cap, const int* __restrict__ iperm,
+                                     const int* __restrict__ lp, int nlev, unsigned* seen, unsigned* res) {
+    for (int q = blockIdx.x; q < nparts; q += gridDim.x) {
+        const int c0 = part_chunk[q], c1 = part_chunk[q + 1];
+        if (c0 < 0 || c1 < c0 || c1 > cap || (q == 0 && c0 != 0)) {
+            if (threadIdx.x == 0) fail(res, 8, q);
+            continue;
+        }
+        for (int c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
+            const int2 k = ch[c];
+            if (k.y < 1 || k.y > 32 || k.x < 0 || k.x > n - k.y) {
+                fail(res, 8, q);
+                continue;
+            }
+            const int l = level_of(k.x, lp, nlev);
+            if (level_of(k.x + k.y - 1, lp, nlev) != l) fail(res, 8, q);
+            if (c > c0 && ch[c - 1].x >= 0 && ch[c - 1].x < n && level_of(ch[c - 1].x, lp, nlev) > l) fail(res, 8, q);
+            for (int r = k.x; r < k.x + k.y; ++r) {
+                const int i = iperm[r];
+                if (i < q * rows || i >= min(n, (q + 1) * rows)) fail(res, 8, q);
+                if (atomicOr(seen + (r >> 5), 1u << (r & 31)) & (1u << (r & 31))) fail(res, 8, q);
+            }
+        }
+    }
+}
+__global__ void k_check_range_cols(int n, int w, int ld, int rows, const unsigned* __restrict__ seen,
+                                   const int* __restrict__ ec, const int* __restrict__ tp, const int* __restrict__ tc,
+                                   const int* __restrict__ oc, const int* __restrict__ otc, const int* __restrict__ iperm,
+                                   unsigned* res) {
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+        if (!((seen[r >> 5] >> (r & 31)) & 1u)) fail(res, 8, r);
+        const int q = iperm[r] / rows;
+        auto code = [&](int c) { return iperm[c] / rows == q ? -2 - (iperm[c] - q * rows) : c; };
+        for (int k = 0; k < w; ++k) {
+            const int c = ec[(long)k * ld + r];
+            if (oc[(long)k * ld + r] != (c < 0 ? -1 : code(c))) fail(res, 8, r);
+        }
+        for (int t = tp[r]; t < tp[r + 1]; ++t)
+            if (otc[t] != code(tc[t])) fail(res, 8, r);
+    }
+}
+
 const char* kCheckName[] = {"", "level map (perm, iperm, level_ptr)", "HEC factor (rows, columns, levels, diagonal)",
                             "chunk table", "partition row map (rowg)", "partitioned factor", "partition chunk table",
-                            "partition tables (part_row, part_chunk)"};
+                            "partition tables (part_row, part_chunk)", "range schedule (chunks, columns)"};
 
 template <typename VT>
 void launch_check_hec(const hec_matrix* T, const int* ec, const void* ev, const int* tp, const int* tc, const void* tv,
@@ -183,6 +230,19 @@ HEC_API hec_status sptrsv_plan_check(const sptrsv_plan* p, void* stream) {
                 p->nchunks[i], p->chunks[i], 32 >> i, 0, n, lv->level_ptr, lv->nlev, nullptr, 3, res);
             count_launch();
         }
+    if (const hec_range_data* R = p->range) {
+        unsigned h = 0;
+        HEC_CUDA(cudaMemcpyAsync(&h, res, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        HEC_CUDA(cudaStreamSynchronize(s));
+        if (h == 0xffffffffu) {  // the map and the factor are sound
+            cudaMemsetAsync(seen, 0, sizeof(unsigned) * ((size_t)(n + 31) / 32), s);
+            k_check_range_chunks<<<R->nparts, 128, 0, s>>>(n, R->nparts, R->rows, R->part_chunk, R->chunks, R->cap_chunks,
+                                                           lv->iperm, lv->level_ptr, lv->nlev, seen, res);
+            k_check_range_cols<<<g, 256, 0, s>>>(n, T->w, T->ld, R->rows, seen, T->ell_col, T->tptr, T->tcol, R->ell_col, R->tcol,
+                                                 lv->iperm, res);
+            count_launch(2);
+        }
+    }
     if (const hec_part_data* P = p->part) {
         cudaMemsetAsync(seen, 0, sizeof(unsigned) * ((size_t)(n + 31) / 32), s);
         k_check_perm<<<g, 256, 0, s>>>(n, P->rowg, seen, res, 4);
@@ -208,6 +268,6 @@ HEC_API hec_status sptrsv_plan_check(const sptrsv_plan* p, void* stream) {
     if (h == 0xffffffffu) return finish(HEC_OK);
     const int check = (int)(h >> 27), where = (int)(h & ((1u << 27) - 1));
     return finish(set_error(HEC_ERR_OUT_OF_BOUNDS, std::string("sptrsv_plan_check: ") +
-                                                       (check > 0 && check < 8 ? kCheckName[check] : "?") +
+                                                       (check > 0 && check < 9 ? kCheckName[check] : "?") +
                                                        " fails at index " + std::to_string(where)));
 }

@@ -122,6 +122,22 @@ struct hec_part_data {
     int* bidx_perm = nullptr;   // [n] plan row -> row of b for sptrsv_lower / sptrsv_upper (iperm[rowg])
 };
 
+// The default schedule of single-right-hand-side sweeps (see sweep.cu, "ranges"): part q owns the
+// original rows [q * rows, (q + 1) * rows).  Inside a level the level order ascends (descends, for an
+// upper factor) in the original row, so a part's rows of a level are consecutive rows of the factor as
+// it is packed, and only a chunk table and the columns in original numbering are added.
+struct hec_range_data {
+    int nparts = 0, rows = 0, threads = 0, cap_chunks = 0;
+    int* ell_col = nullptr;     // [w * ld] the slab's columns: -1 empty, -2 - s word s of the range, else the row
+    int* tcol = nullptr;        // [tail_nnz] the tail's
+    int2* chunks = nullptr;     // (first level-ordered row, rows <= 32), part by part in level order
+    int* part_chunk = nullptr;  // [nparts + 1]
+    void* xpb[2] = {nullptr, nullptr};  // level-ordered solution words: a sweep polls one and sets the other
+                                        // to the sentinel
+    int* state = nullptr;       // [2] which of the two, and the blocks that have finished; kept on the device, so
+                                // that a captured sweep can be replayed
+};
+
 struct sptrsv_plan {
     hec_part_data* part = nullptr;  // set by sptrsv_plan_partition
     const hec_matrix* T = nullptr;
@@ -137,6 +153,8 @@ struct sptrsv_plan {
     int nchunks[5] = {};
     void* dinv = nullptr;      // reciprocal diagonal in the work type (NULL: the kernel divides)
     int lpr1 = 1;              // lanes per row of single-right-hand-side sweeps (1, 2, 4 or 8)
+    hec_range_data* range = nullptr;  // NULL: not built (see build_range)
+    int use_range = 1;         // single-right-hand-side sweeps without a partition take the ranges
     int use_part = 1;          // single-right-hand-side sweeps take the partition when there is one
 };
 

@@ -834,10 +834,11 @@ struct DepSlots {
         unsigned pend = cross;
         for (unsigned it = 1; __any_sync(kFull, pend != 0u); ++it) {
 #pragma unroll
-            for (int k = 0; k < NS; ++k) ld_relaxed_if((pend >> k) & 1u, xp + col[k], raw[k]);
+            for (int k = 0; k < NS; ++k)
+                if ((pend >> k) & 1u) raw[k] = W::load(xp + col[k]);
 #pragma unroll
             for (int k = 0; k < NS; ++k)
-                if (raw[k] != W::kSent) pend &= ~(1u << k);
+                if (((pend >> k) & 1u) && raw[k] != W::kSent) pend &= ~(1u << k);
             if (give_up(it)) break;
         }
         WT lw[NS];
@@ -1085,6 +1086,202 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_part(PartParams p) {
     for (int i = threadIdx.x; i < hi - lo; i += blockDim.x) nxp[lo + i] = W::kSent;
 }
 
+// ---- ranges: the default schedule of single-right-hand-side sweeps -----------------------------
+// The partitioned idea without a caller's partition and without a second copy of the factor: part q
+// is the range [q * rows, (q + 1) * rows) of original rows, one resident block each, its solution in
+// shared memory at (original row - q * rows).  Inside a level the level order follows the original row,
+// so a range's rows of a level are consecutive rows of the packed factor: the kernel reads the slab as
+// it is, and needs only its own chunk table and the columns coded by where their words are: -2 - s for
+// word s of the range's shared solution, the level-ordered row for a row of another range, whose word
+// is polled in global memory (level order keeps a chunk's words in a few sectors).
+// Every row adds its entries in the order of k_sweep, so results are the same bit for bit.
+//   What bounds it is the latency of a level, as in the other sweeps: about 0.5 us where k_sweep takes 1
+// (its producers and consumers meet in L2).  Index loads run a chunk ahead of the row's loads, which
+// for FP32 work run a chunk ahead of its wait.
+//   Both word buffers and the flag that says which one this sweep polls live on the device: the block
+// that finishes last turns the flag, so no fill launch is needed and a captured graph can be replayed.
+struct RangeParams {
+    int n, ld, w, rows;
+    const int* __restrict__ ell_col;  // coded (see above)
+    const void* __restrict__ ell_val;
+    const int* __restrict__ tptr;
+    const int* __restrict__ tcol;     // coded
+    const void* __restrict__ tval;
+    const void* __restrict__ dinv;
+    const int* __restrict__ iperm;
+    const int* __restrict__ part_chunk;
+    const int2* __restrict__ chunks;
+    const double* __restrict__ b;
+    int ldb;
+    const int* __restrict__ gather;
+    double* __restrict__ x;
+    int ldx;
+    const int* __restrict__ scatter;
+    void* xpb[2];
+    int* state;
+    int* status;
+    long long budget;
+    int skip_row;
+    int b32, x32;
+};
+
+// of one lane's row: its original number, the row of b it reads, the row of x it writes (-1: none)
+struct RangeIdx {
+    int id, gr, sr;
+    __device__ __forceinline__ void load(const RangeParams& p, int2 ch, int lane) {
+        id = sr = -1;
+        gr = 0;
+        if (lane < ch.y) {
+            const int r = ch.x + lane;
+            id = __ldg(p.iperm + r);
+            gr = p.gather == p.iperm ? id : p.gather ? __ldg(p.gather + r) : r;
+            sr = p.scatter == p.iperm ? id : p.scatter ? __ldg(p.scatter + r) : r;
+        }
+    }
+};
+
+template <typename VT, typename XT, typename AT, int NP>
+struct RangeRow {
+    AT b;
+    XT d;
+    int t0, t1;
+    int cc[NP];
+    VT v[NP];
+    __device__ __forceinline__ void load(const RangeParams& p, int2 ch, int lane, int gr) {
+        b = AT(0);
+        d = XT(1);
+        t0 = 0;
+        t1 = 1;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            cc[k] = -1;
+            v[k] = VT(0.0f);
+        }
+        if (lane < ch.y) {
+            const int r = ch.x + lane;
+            b = ld_rhs<AT>(p.b, p.b32, (long)gr * p.ldb);
+            t0 = __ldg(p.tptr + r);
+            t1 = __ldg(p.tptr + r + 1);
+            d = __ldg((const XT*)p.dinv + r);
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                if (k < p.w) {
+                    const long s = (long)k * p.ld + r;
+                    cc[k] = __ldg(p.ell_col + s);
+                    v[k] = __ldg((const VT*)p.ell_val + s);
+                }
+            }
+        }
+    }
+};
+
+template <typename XT, typename AT, int NS>
+__device__ __forceinline__ void range_set(DepSlots<XT, AT, NS>& d, int k, unsigned int sbase, int cc, AT v) {
+    if (cc < -1) d.set_local(k, sbase + (unsigned int)(-2 - cc) * (unsigned int)sizeof(XT), v);
+    else if (cc >= 0) d.set_cross(k, cc, v);
+}
+template <typename XT, typename AT, int NS>
+__device__ __forceinline__ void range_set(DepBatchP<XT, AT, NS>& d, int k, unsigned int sbase, int cc, AT v) {
+    if (cc < -1) d.set(k, sbase, -2 - cc, 0, 0x7fffffff, v);  // in [0, ...): local
+    else if (cc >= 0) d.set(k, sbase, cc, 1, 0, v);           // in no range: global
+}
+
+template <typename VT, typename XT, int WMAX>
+__global__ void __launch_bounds__(1024, 1) k_sweep_range(RangeParams p) {
+    typedef typename Acc<XT>::T AT;
+    typedef Word<XT> W;
+    typedef typename W::T WT;
+    constexpr bool PF = sizeof(AT) == 4 && WMAX <= 4;  // a second row in registers (64 a thread) only where it fits
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    WT* sxp = (WT*)smem_raw;
+    const unsigned int sbase = (unsigned int)__cvta_generic_to_shared(smem_raw);
+    const int lo = blockIdx.x * p.rows, hi = min(p.n, lo + p.rows);
+    const int turn = __ldcg(p.state);  // turned by the last block to finish, when every block has read it
+    for (int i = threadIdx.x; i < hi - lo; i += blockDim.x) sxp[i] = W::kSent;
+    __syncthreads();
+    const int c0 = __ldg(p.part_chunk + blockIdx.x), c1 = __ldg(p.part_chunk + blockIdx.x + 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const VT* __restrict__ ev = (const VT*)p.ell_val;
+    const VT* __restrict__ tv = (const VT*)p.tval;
+    XT* xp = (XT*)p.xpb[turn];
+    auto chunk = [&](int c) { return c < c1 ? __ldg(p.chunks + c) : make_int2(0, 0); };
+    int c = c0 + warp;
+    int2 ch = chunk(c), ch1 = chunk(c + nwarps), ch2 = chunk(c + 2 * nwarps);
+    RangeIdx ix, ix1;
+    ix.load(p, ch, lane);
+    ix1.load(p, ch1, lane);
+    RangeRow<VT, XT, AT, WMAX> row, nxt;
+    if (PF) nxt.load(p, ch, lane, ix.gr);
+    for (; c < c1; c += nwarps) {
+        RangeIdx ix2;
+        if (PF) {
+            row = nxt;
+            nxt.load(p, ch1, lane, ix1.gr);
+        } else {
+            row.load(p, ch, lane, ix.gr);
+        }
+        ix2.load(p, ch2, lane);
+        const int2 ch3 = chunk(c + 3 * nwarps);
+        const int r = ch.x + lane;
+        const bool act = lane < ch.y;
+        AT acc = row.b;
+        const AT diag = (AT)row.d;
+        const int t0 = row.t0, tl = row.t1 - 1 - row.t0;
+        typename SlabDeps<XT, AT, WMAX>::T slab;
+        slab_clear(slab, sbase);
+#pragma unroll
+        for (int k = 0; k < WMAX; ++k) range_set(slab, k, sbase, row.cc[k], widen_v<VT, AT>(row.v[k]));
+        const int tmax = __reduce_max_sync(kFull, tl);
+        slab_wait(slab, xp, p.status, p.budget);
+        acc = slab.accumulate(acc, p.w);
+        for (int kb = WMAX; kb < p.w; kb += kTailBatch) {  // wider slabs, kTailBatch slots at a time
+            DepBatchP<XT, AT, kTailBatch> more;
+            more.clear();
+#pragma unroll
+            for (int j = 0; j < kTailBatch; ++j) {
+                const int k = kb + j;
+                if (act && k < p.w) {
+                    const long s = (long)k * p.ld + r;
+                    range_set(more, j, sbase, __ldg(p.ell_col + s), ldv<VT, AT>(ev + s));
+                }
+            }
+            more.poll(xp);
+            more.wait(xp, p.status, p.budget);
+            acc = more.accumulate(acc);
+        }
+        for (int tb = 0; tb < tmax; tb += kTailBatch) {
+            DepBatchP<XT, AT, kTailBatch> tail;
+            tail.clear();
+#pragma unroll
+            for (int k = 0; k < kTailBatch; ++k)
+                if (tb + k < tl)
+                    range_set(tail, k, sbase, __ldg(p.tcol + t0 + tb + k), ldv<VT, AT>(tv + t0 + tb + k));
+            tail.poll(xp);
+            tail.wait(xp, p.status, p.budget);
+            acc = tail.accumulate(acc);
+        }
+        const AT xr = acc * diag;
+        if (act && r != p.skip_row) {
+            WT wv = sizeof(XT) == 8 ? (WT)__double_as_longlong((double)(XT)xr) : (WT)__float_as_uint((float)(XT)xr);
+            if (wv == W::kSent) wv = sizeof(XT) == 8 ? (WT)0x7FF8000000000000ull : (WT)0x7FC00000u;
+            *(volatile WT*)(sxp + (ix.id - lo)) = wv;  // consumers in this range
+            publish_x(xp + r, (XT)xr);                 // consumers in other ranges
+        }
+        if (act && ix.sr >= 0) st_sol(p.x, p.x32, (long)ix.sr * p.ldx, xr);
+        ch = ch1;
+        ch1 = ch2;
+        ch2 = ch3;
+        ix = ix1;
+        ix1 = ix2;
+    }
+    WT* nxp = (WT*)p.xpb[turn ^ 1];  // what the next sweep polls: any split over the blocks does
+    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) nxp[i] = W::kSent;
+    if (threadIdx.x == 0 && atomicAdd(p.state + 1, 1) == (int)gridDim.x - 1) {
+        p.state[1] = 0;
+        p.state[0] = turn ^ 1;
+    }
+}
+
 template <typename XT>
 __global__ void k_fill_sentinel(XT* xp, long count) {
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1330,6 +1527,21 @@ const void* part_kernel(int w) {
 }
 }  // namespace
 
+namespace {
+template <typename VT, typename XT>
+const void* range_kernel(int w) {
+    return w <= 3   ? (const void*)k_sweep_range<VT, XT, 3>
+           : w <= 4 ? (const void*)k_sweep_range<VT, XT, 4>
+                    : (const void*)k_sweep_range<VT, XT, 8>;
+}
+const void* range_kernel(const hec_matrix* T) {
+    return T->vdt == HEC_F64 ? range_kernel<double, double>(T->w)
+           : T->vdt == HEC_F32 ? range_kernel<float, float>(T->w)
+                               : range_kernel<__nv_bfloat16, float>(T->w);
+}
+constexpr size_t kRangeSmem = 227 * 1024;  // shared solution of one block
+}  // namespace
+
 hec_status sweep(const sptrsv_plan* pl, int nrhs, const double* b, int ldb, const int* gather, double* x, int ldx,
                  const int* scatter, cudaStream_t s, bool b32, bool x32, const int* bidx, bool bplan) {
     const hec_matrix* T = pl->T;
@@ -1371,6 +1583,45 @@ hec_status sweep(const sptrsv_plan* pl, int nrhs, const double* b, int ldb, cons
             case HEC_F32: return dispatch_part<float, float>(pl, pp, s);
             default: return dispatch_part<__nv_bfloat16, float>(pl, pp, s);
         }
+    }
+    if (pl->range && pl->use_range && nrhs == 1 && pl->lpr1 == 1) {
+        const hec_range_data* R = pl->range;
+        RangeParams rp;
+        rp.n = T->n;
+        rp.ld = T->ld;
+        rp.w = T->w;
+        rp.rows = R->rows;
+        rp.ell_col = R->ell_col;
+        rp.ell_val = T->ell_val;
+        rp.tptr = T->tptr;
+        rp.tcol = R->tcol;
+        rp.tval = T->tval;
+        rp.dinv = pl->dinv;
+        rp.iperm = pl->lv->iperm;
+        rp.part_chunk = R->part_chunk;
+        rp.chunks = R->chunks;
+        rp.b = b;
+        rp.ldb = ldb;
+        rp.gather = gather;
+        rp.x = x;
+        rp.ldx = ldx;
+        rp.scatter = scatter;
+        rp.xpb[0] = R->xpb[0];
+        rp.xpb[1] = R->xpb[1];
+        rp.state = R->state;
+        rp.status = pl->status;
+        rp.budget = pl->wait_cycles;
+        rp.skip_row = pl->skip_row;
+        rp.b32 = b32;
+        rp.x32 = x32;
+        void* args[] = {&rp};
+        void* tok = nullptr;
+        profile_begin(s, &tok);
+        HEC_CUDA(cudaLaunchCooperativeKernel(range_kernel(T), dim3(R->nparts), dim3(R->threads), args,
+                                             (size_t)R->rows * work_size(T->vdt), s));
+        profile_end(s, tok);
+        count_launch();
+        return HEC_OK;
     }
     SweepParams sp;
     sp.n = T->n;
@@ -1449,8 +1700,16 @@ void free_part(hec_part_data* P) {
     delete P;
 }
 
+void free_range(hec_range_data* R) {
+    if (!R) return;
+    dfree(R->ell_col); dfree(R->tcol); dfree(R->chunks); dfree(R->part_chunk);
+    dfree(R->xpb[0]); dfree(R->xpb[1]); dfree(R->state);
+    delete R;
+}
+
 void free_plan(sptrsv_plan* p) {
     if (!p) return;
+    free_range(p->range);
     dfree(p->xp);
     dfree(p->status);
     for (int i = 0; i < 5; ++i) dfree(p->chunks[i]);
@@ -1737,6 +1996,180 @@ hec_status build_partition(sptrsv_plan* p, const int* part, int nparts, cudaStre
     return done(HEC_OK);
 }
 
+namespace {
+// the columns of slab and tail coded by where their words are (see RangeParams); *ncross: entries whose
+// row is in another range
+__global__ void k_range_cols(int n, int ld, int w, int rows, const int* __restrict__ ec, const int* __restrict__ tp,
+                             const int* __restrict__ tc, const int* __restrict__ iperm, int* oec, int* otc,
+                             unsigned long long* ncross) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    int cross = 0;
+    if (r < n) {
+        const int q = __ldg(iperm + r) / rows;
+        auto code = [&](int c) {
+            const int j = __ldg(iperm + c);
+            if (j / rows == q) return -2 - (j - q * rows);
+            ++cross;
+            return c;
+        };
+        for (int k = 0; k < w; ++k) {
+            const long s = (long)k * ld + r;
+            const int c = __ldg(ec + s);
+            oec[s] = c >= 0 ? code(c) : -1;
+        }
+        for (int t = __ldg(tp + r); t < __ldg(tp + r + 1); ++t) otc[t] = code(__ldg(tc + t));
+    } else if (r < ld) {
+        for (int k = 0; k < w; ++k) oec[(long)k * ld + r] = -1;
+    }
+    cross = __reduce_add_sync(0xffffffffu, cross);
+    if ((threadIdx.x & 31) == 0 && cross) atomicAdd(ncross, (unsigned long long)cross);
+}
+// first row in [a, b) of a level whose original number, ascending (descending for an upper factor), has
+// reached v
+__device__ __forceinline__ int range_bound(const int* __restrict__ iperm, int a, int b, int v, int uplo) {
+    while (a < b) {
+        const int mid = (a + b) >> 1;
+        const int i = __ldg(iperm + mid);
+        if (uplo ? i >= v : i < v) a = mid + 1; else b = mid;
+    }
+    return a;
+}
+// (part q, level l) at q * nlev + l: its chunks of at most 32 rows, counted (chunks == NULL, into pos;
+// nseg counts the nonempty ones, most[l] the most of a part) or written from pos
+__global__ void k_range_chunks(int n, int nlev, int nparts, int rows, int uplo, const int* __restrict__ iperm,
+                               const int* __restrict__ level_ptr, int* pos, int2* chunks, int* part_chunk,
+                               int* most, unsigned long long* nseg) {
+    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= (long)nparts * nlev) return;
+    const int q = (int)(k / nlev), l = (int)(k - (long)q * nlev);
+    const int a = __ldg(level_ptr + l), b = __ldg(level_ptr + l + 1);
+    const int lo = q * rows, hi = min(n, lo + rows);  // original rows of the part
+    const int r0 = range_bound(iperm, a, b, uplo ? hi : lo, uplo), r1 = range_bound(iperm, r0, b, uplo ? lo : hi, uplo);
+    if (!chunks) {
+        const int cnt = (r1 - r0 + 31) / 32;
+        pos[k] = cnt;
+        if (cnt) {
+            atomicAdd(nseg, 1ull);
+            atomicMax(most + l, cnt);
+        }
+        return;
+    }
+    int c = pos[k];
+    if (l == 0) part_chunk[q] = c;
+    if (k == (long)nparts * nlev - 1) part_chunk[nparts] = pos[k + 1];
+    for (int r = r0; r < r1; r += 32, ++c) chunks[c] = make_int2(r, min(32, r1 - r));
+}
+// estimated time of both schedules, summed over the levels, in units of 10 ns: a level takes the latency of
+// its hand-off or, when longer, the chunks of the block that has the most of them (ranges) or of an SM's
+// share (global).  cost[0] ranges, cost[1] global.
+__global__ void k_range_cost(int nlev, int sms, const int* __restrict__ level_ptr, const int* __restrict__ most,
+                             unsigned long long* cost) {
+    constexpr int kHop = 45, kChunk = 12, kGlobalHop = 85, kGlobalChunk = 16;
+    unsigned a = 0, b = 0;
+    for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlev; l += gridDim.x * blockDim.x) {
+        a += max(kHop, kChunk * most[l]);
+        b += max(kGlobalHop, kGlobalChunk * ((level_ptr[l + 1] - level_ptr[l] + 31) / 32) / sms);
+    }
+    a = __reduce_add_sync(0xffffffffu, a);
+    b = __reduce_add_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(cost, (unsigned long long)a);
+        atomicAdd(cost + 1, (unsigned long long)b);
+    }
+}
+}  // namespace
+
+// The range schedule of a plan, when it pays and fits: a lane per row, the solution in the shared memory
+// of at most one block an SM, levels not so many that the (part, level) table outgrows the factor, at
+// most 60 % of the entries in another range (they would still meet in L2), and an estimated time at
+// least 15 % below the global schedule's (k_range_cost: a range whose level is many chunks is bound by
+// its one SM; its constants are fits to the times below).
+//   Parts: kRangeLevelRows rows of an average level each.  More parts cross more boundaries on the
+// dependency chain, fewer make a level's chunks queue in a block (24 / 43 / 64 rows: 50^3 151 / 129 / 151 us,
+// 100^3 457 / 359 / 341, 128^3 512 / 487 / 484).
+// L+U apply of ILU(0), global / range schedule, FP64 (FP32): 5-point 64 x 64 166 / 79 us (132 / 60),
+// 150 x 150 374 / 185 (313 / 128), 1000 x 1000 2810 / 1190 (2250 / 885); 7-point 16^3 80 / 42 (58 / 30),
+// 31 x 37 x 29 161 / 80 (130 / 62), 50^3 245 / 129 (191 / 102), 64^3 323 / 172 (244 / 136), 100^3 548 / 359
+// (423 / 290), 128^3 723 / 486 (542 / 413), 160^3 937 / 726 (684 / 580); 576 Schwarz boxes of 128^3
+// 201 / 162 (177 / 116).  Where the estimate keeps the global one: 64 boxes 239 / 357 (193 / 270), FP32
+// 200^3 (921 / 926), random rows of six entries 248 / 390.
+hec_status build_range(sptrsv_plan* p) {
+    constexpr int kRangeLevelRows = 43;
+    const hec_matrix* T = p->T;
+    const hec_levels* lv = p->lv;
+    const int n = T->n, nlev = lv->nlev, sms = num_sms();
+    if (n == 0 || p->lpr1 != 1 || sms == 0) return HEC_OK;
+    const size_t ws = work_size(T->vdt);
+    const long avg = (n + nlev - 1) / nlev;
+    long need = (long)((ws * (size_t)n + kRangeSmem - 1) / kRangeSmem);
+    long parts = std::max(need, std::min((avg + kRangeLevelRows / 2) / kRangeLevelRows, (long)sms));
+    parts = std::max(1L, std::min(parts, (long)n));
+    if (parts > sms || parts * nlev > 4L * n + 1024) return HEC_OK;
+    hec_range_data* R = new hec_range_data();
+    R->rows = (int)((n + parts - 1) / parts);
+    R->nparts = (n + R->rows - 1) / R->rows;
+    int *pos = nullptr, *most = nullptr;
+    unsigned long long* counts = nullptr;  // nonempty (part, level) pairs; entries in another range; costs
+    hec_status st = HEC_OK;
+    cudaStream_t s = 0;
+    auto done = [&](hec_status e) {
+        dfree(pos); dfree(most); dfree(counts);
+        if (e != HEC_OK) free_range(R);
+        if (e == HEC_ERR_OOM) {  // no room: the plan keeps the global schedule
+            clear_error();
+            return HEC_OK;
+        }
+        return e;
+    };
+    const long tbl = (long)R->nparts * nlev;
+    if ((size_t)R->rows * ws > kRangeSmem ||
+        cudaFuncSetAttribute(range_kernel(T), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRangeSmem) != cudaSuccess) {
+        cudaGetLastError();
+        free_range(R);
+        return HEC_OK;
+    }
+    R->cap_chunks = (int)std::min((long)n, tbl + n / 32);
+    if ((st = dalloc(&pos, (size_t)tbl + 1)) || (st = dalloc(&most, (size_t)nlev)) || (st = dalloc(&counts, 4)) || (st = dalloc(&R->chunks, (size_t)R->cap_chunks)) ||
+        (st = dalloc(&R->part_chunk, (size_t)R->nparts + 1)) || (st = dalloc(&R->ell_col, (size_t)T->w * T->ld)) ||
+        (st = dalloc(&R->tcol, (size_t)T->tail_nnz)) || (st = dmalloc(&R->xpb[0], ws * (size_t)n + 16)) ||
+        (st = dmalloc(&R->xpb[1], ws * (size_t)n + 16)) || (st = dalloc(&R->state, 2)))
+        return done(st);
+    if (cudaMemsetAsync(R->state, 0, 2 * sizeof(int), s) != cudaSuccess || cudaMemsetAsync(counts, 0, 4 * sizeof(*counts), s) != cudaSuccess ||
+        cudaMemsetAsync(most, 0, sizeof(int) * (size_t)nlev, s) != cudaSuccess)
+        return done(cuda_error(cudaGetLastError(), "memset"));
+    const int g = (int)((tbl + 127) / 128);
+    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, lv->uplo, lv->iperm, lv->level_ptr, pos, nullptr, nullptr,
+                                     most, counts);
+    k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, lv->level_ptr, most, counts + 2);
+    if ((st = exclusive_scan_i32(pos, pos, (int)tbl, true, s))) return done(st);
+    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, lv->uplo, lv->iperm, lv->level_ptr, pos, R->chunks,
+                                     R->part_chunk, most, counts);
+    k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, T->ell_col, T->tptr, T->tcol, lv->iperm,
+                                                     R->ell_col, R->tcol, counts + 1);
+    const int fb = std::min(4096, (n + 255) / 256);  // the words of the first sweep; each sweep sets its successor's
+    if (ws == 8) k_fill_sentinel<double><<<fb, 256, 0, s>>>((double*)R->xpb[0], n);
+    else k_fill_sentinel<float><<<fb, 256, 0, s>>>((float*)R->xpb[0], n);
+    count_launch(5);
+    unsigned long long h[4] = {0, 0, 0, 0};
+    if (cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return done(cuda_error(cudaGetLastError(), "range schedule"));
+    // threads: 16 warps hold a few levels of a part's chunks; a factor too large for the caches needs its rows
+    // loaded further ahead (L+U apply with 512 / 1024 threads: 64 x 64 grid FP32 57.8 / 70.5 us; FP64: 400 x 300
+    // 409 / 506, 1000 x 1000 1187 / 1488, 64^3 172 / 195, 100^3 392 / 359, 128^3 543 / 486)
+    const long long nnz_bound = (long long)T->w * n + T->tail_nnz;
+    const int seg_rows = n / (int)std::max(1ull, h[0]);
+    R->threads = seg_rows >= 40 && n >= 500000 ? 1024 : 512;
+    const long long entries = nnz_bound - n;  // off-diagonals and padding
+    if ((long long)h[1] * 10 > entries * 6 || h[2] * 100 > h[3] * 85 ||
+        max_coop_blocks(range_kernel(T), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
+        free_range(R);
+        R = nullptr;
+    }
+    p->range = R;
+    return done(HEC_OK);
+}
+
 // resident blocks of the partitioned kernel for `smem` bytes of shared solution per block
 int part_capacity(const sptrsv_plan* p, int threads, size_t smem) {
     const void* k = p->T->vdt == HEC_F64 ? part_kernel<double, double>(p->T->w)
@@ -1788,6 +2221,9 @@ HEC_API hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* l
     for (int k = 1; k <= max_nrhs; ++k) needed |= 1u << log2i(sweep_lpr(k, tri->vdt));
     if (st == HEC_OK) st = build_chunks(p, needed);
     if (st == HEC_OK) st = build_dinv(p);
+    // a launch shape or lane layout asked for by the caller is that of the global kernels
+    const bool shaped = tune && (tune->block_threads || tune->blocks_per_sm || tune->backoff_ns || tune->lanes_per_row);
+    if (st == HEC_OK && max_nrhs == 1 && !shaped) st = build_range(p);
     if (st != HEC_OK) { free_plan(p); return st; }
     *out = p;
     return HEC_OK;
@@ -1870,8 +2306,8 @@ HEC_API hec_status sptrsv_upper(const sptrsv_plan* p, int nrhs, const double* b,
 //  - for one right-hand side, lanes per row (1, 2, 4 or 8): one lane per row (thread per row)
 //    against several lanes sharing a row's dependencies and a shuffle reduction (the
 //    thread-versus-warp choice by row length);
-//  - for one right-hand side on a plan given a partition, the partitioned schedule against the
-//    best global one.
+//  - for one right-hand side, the range schedule (when the plan has it), and on a plan given a
+//    partition the partitioned schedule, against the best global one.
 // The point-to-point sweep has no per-level barriers, so the paper's level-merging threshold has
 // no counterpart.  Results are cached per matrix signature (rows, slab width, tail entries,
 // levels, value type, right-hand sides, whether a partition was given) so identical factors are
@@ -1892,7 +2328,7 @@ struct TuneKeyHash {
     }
 };
 struct TuneChoice {
-    int threads, blocks, lpr1, use_part;
+    int threads, blocks, lpr1, use_part, use_range;
 };
 std::mutex g_tune_mu;
 std::unordered_map<TuneKey, TuneChoice, TuneKeyHash> g_tune_cache;
@@ -1902,6 +2338,7 @@ void apply_choice(sptrsv_plan* p, const TuneChoice& c, hec_tune* out) {
     p->blocks = c.blocks;
     p->lpr1 = c.lpr1;
     p->use_part = c.use_part;
+    p->use_range = c.use_range;
     if (out) {
         *out = hec_tune{};
         out->block_threads = c.threads;
@@ -1940,7 +2377,7 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const TuneChoice saved{p->threads, p->blocks, p->lpr1, p->use_part};
+    const TuneChoice saved{p->threads, p->blocks, p->lpr1, p->use_part, p->use_range};
     // one warm-up and three timed sweeps of the plan as it is set
     auto time_it = [&](float* ms) -> hec_status {
         hec_status r = sweep(p, nrhs, b, nrhs, p->lv->iperm, x, nrhs, p->lv->iperm, s);
@@ -1964,7 +2401,7 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
         for (int ti = 0; ti < 2 && st == HEC_OK; ++ti) {
             for (int bi = 0; bi < 4 && st == HEC_OK; ++bi) {
                 if (cand_t[ti] * cand_b[bi] > 2048) continue;
-                const TuneChoice c{cand_t[ti], cand_b[bi], lpr, 0};
+                const TuneChoice c{cand_t[ti], cand_b[bi], lpr, 0, 0};
                 apply_choice(p, c, nullptr);
                 float ms = 0.f;
                 st = time_it(&ms);
@@ -1972,8 +2409,15 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
             }
         }
     }
+    if (st == HEC_OK && nrhs == 1 && p->range) {  // the range schedule (its launch shape is its own)
+        const TuneChoice c{bc.threads, bc.blocks, saved.lpr1, 0, 1};
+        apply_choice(p, c, nullptr);
+        float ms = 0.f;
+        st = time_it(&ms);
+        if (st == HEC_OK && ms < best) { best = ms; bc = c; }
+    }
     if (st == HEC_OK && parted) {  // the partitioned schedule (its launch shape is the partition's)
-        const TuneChoice c{bc.threads, bc.blocks, bc.lpr1, 1};
+        const TuneChoice c{bc.threads, bc.blocks, bc.lpr1, 1, bc.use_range};
         apply_choice(p, c, nullptr);
         float ms = 0.f;
         st = time_it(&ms);
