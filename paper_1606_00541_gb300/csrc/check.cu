@@ -138,7 +138,7 @@ __global__ void k_check_part_chunks(int nparts, const int* __restrict__ part_row
 // the range schedule: every row in exactly one chunk (`seen`), of its range and of one level, a range's
 // chunks in level order; the columns those of the factor in original numbering
 __global__ void k_check_range_chunks(int n, int nparts, int rows, const int* __restrict__ part_chunk,
-                                     const int2* __restrict__ ch, int cap, const int* __restrict__ iperm,
+                                     const int2* __restrict__ ch, int cap, int rpw, const int* __restrict__ iperm,
                                      const int* __restrict__ lp, int nlev, unsigned* seen, unsigned* res) {
     for (int q = blockIdx.x; q < nparts; q += gridDim.x) {
         const int c0 = part_chunk[q], c1 = part_chunk[q + 1];
@@ -148,7 +148,7 @@ __global__ void k_check_range_chunks(int n, int nparts, int rows, const int* __r
         }
         for (int c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
             const int2 k = ch[c];
-            if (k.y < 1 || k.y > 32 || k.x < 0 || k.x > n - k.y) {
+            if (k.y < 1 || k.y > rpw || k.x < 0 || k.x > n - k.y) {
                 fail(res, 8, q);
                 continue;
             }
@@ -236,7 +236,7 @@ HEC_API hec_status sptrsv_plan_check(const sptrsv_plan* p, void* stream) {
         HEC_CUDA(cudaStreamSynchronize(s));
         if (h == 0xffffffffu) {  // the map and the factor are sound
             cudaMemsetAsync(seen, 0, sizeof(unsigned) * ((size_t)(n + 31) / 32), s);
-            k_check_range_chunks<<<R->nparts, 128, 0, s>>>(n, R->nparts, R->rows, R->part_chunk, R->chunks, R->cap_chunks,
+            k_check_range_chunks<<<R->nparts, 128, 0, s>>>(n, R->nparts, R->rows, R->part_chunk, R->chunks, R->cap_chunks, 32 / R->lanes,
                                                            lv->iperm, lv->level_ptr, lv->nlev, seen, res);
             k_check_range_cols<<<g, 256, 0, s>>>(n, T->w, T->ld, R->rows, seen, T->ell_col, T->tptr, T->tcol, R->ell_col, R->tcol,
                                                  lv->iperm, res);

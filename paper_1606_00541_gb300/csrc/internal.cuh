@@ -128,9 +128,11 @@ struct hec_part_data {
 // it is packed, and only a chunk table and the columns in original numbering are added.
 struct hec_range_data {
     int nparts = 0, rows = 0, threads = 0, cap_chunks = 0;
+    int lanes = 1;              // lanes per row: chunks hold up to 32 / lanes rows
+    int virt = 1;               // lanes per row of the global kernel whose sums it reproduces
     int* ell_col = nullptr;     // [w * ld] the slab's columns: -1 empty, -2 - s word s of the range, else the row
     int* tcol = nullptr;        // [tail_nnz] the tail's
-    int2* chunks = nullptr;     // (first level-ordered row, rows <= 32), part by part in level order
+    int2* chunks = nullptr;     // (first level-ordered row, rows), part by part in level order
     int* part_chunk = nullptr;  // [nparts + 1]
     void* xpb[2] = {nullptr, nullptr};  // level-ordered solution words: a sweep polls one and sets the other
                                         // to the sentinel

@@ -842,6 +842,19 @@ struct DepSlots {
             if (give_up(it)) break;
         }
         WT lw[NS];
+        if (NS > 4) {
+            // many slots: the waiting warps' polls would fill the shared-memory pipe, so a lane first spins on
+            // its last local word alone (slots ascend in level order: the highest level of the row)
+            unsigned int last = addr[0];
+#pragma unroll
+            for (int k = 0; k < NS; ++k)
+                if ((local >> k) & 1u) last = addr[k];
+            for (unsigned it = 1;; ++it) {
+                const WT w = sizeof(WT) == 8 ? (WT)ld_shared_u64(last) : (WT)ld_shared_u32(last);
+                if (__all_sync(kFull, w != W::kSent || local == 0u)) break;
+                if (give_up(it)) break;
+            }
+        }
         for (unsigned it = 1;; ++it) {
             bool ok = true;
 #pragma unroll
@@ -1128,11 +1141,11 @@ struct RangeParams {
 // of one lane's row: its original number, the row of b it reads, the row of x it writes (-1: none)
 struct RangeIdx {
     int id, gr, sr;
-    __device__ __forceinline__ void load(const RangeParams& p, int2 ch, int lane) {
+    __device__ __forceinline__ void load(const RangeParams& p, int2 ch, int rsub) {
         id = sr = -1;
         gr = 0;
-        if (lane < ch.y) {
-            const int r = ch.x + lane;
+        if (rsub < ch.y) {
+            const int r = ch.x + rsub;
             id = __ldg(p.iperm + r);
             gr = p.gather == p.iperm ? id : p.gather ? __ldg(p.gather + r) : r;
             sr = p.scatter == p.iperm ? id : p.scatter ? __ldg(p.scatter + r) : r;
@@ -1187,7 +1200,7 @@ __device__ __forceinline__ void range_set(DepBatchP<XT, AT, NS>& d, int k, unsig
 }
 
 template <typename VT, typename XT, int WMAX>
-__global__ void __launch_bounds__(1024, 1) k_sweep_range(RangeParams p) {
+__global__ void __launch_bounds__(WMAX <= 4 ? 1024 : 512, 1) k_sweep_range(RangeParams p) {
     typedef typename Acc<XT>::T AT;
     typedef Word<XT> W;
     typedef typename W::T WT;
@@ -1227,12 +1240,12 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_range(RangeParams p) {
         AT acc = row.b;
         const AT diag = (AT)row.d;
         const int t0 = row.t0, tl = row.t1 - 1 - row.t0;
-        typename SlabDeps<XT, AT, WMAX>::T slab;
-        slab_clear(slab, sbase);
+        DepSlots<XT, AT, WMAX> slab;
+        slab.clear(sbase);
 #pragma unroll
         for (int k = 0; k < WMAX; ++k) range_set(slab, k, sbase, row.cc[k], widen_v<VT, AT>(row.v[k]));
         const int tmax = __reduce_max_sync(kFull, tl);
-        slab_wait(slab, xp, p.status, p.budget);
+        slab.wait(xp, p.status, p.budget);
         acc = slab.accumulate(acc, p.w);
         for (int kb = WMAX; kb < p.w; kb += kTailBatch) {  // wider slabs, kTailBatch slots at a time
             DepBatchP<XT, AT, kTailBatch> more;
@@ -1275,6 +1288,115 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_range(RangeParams p) {
         ix1 = ix2;
     }
     WT* nxp = (WT*)p.xpb[turn ^ 1];  // what the next sweep polls: any split over the blocks does
+    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) nxp[i] = W::kSent;
+    if (threadIdx.x == 0 && atomicAdd(p.state + 1, 1) == (int)gridDim.x - 1) {
+        p.state[1] = 0;
+        p.state[0] = turn ^ 1;
+    }
+}
+
+// Long rows in the range schedule.  The global kernel shares such a row among V = 2, 4 or 8 lanes
+// (k_sweep_lpr); its sums are V partial sums, partial sum v over the slots and tail entries v, v + V, ...,
+// added by a butterfly.  Here two lanes compute the same V partial sums, lane h those with v % 2 == h, and
+// add them in the butterfly's pairs, so results are the same bit for bit.  Two lanes instead of eight
+// because an FP64 instruction costs the SM 16 cycles whatever its lanes do: a warp's FMAs then serve 16
+// rows, and the V / 2 chains of a lane overlap.  Needs w <= 3 V (the slots k_sweep_lpr takes before the
+// tail) and rows of up to 2 NS slots wait once.
+template <typename VT, typename XT, int V, int NS>
+__global__ void __launch_bounds__(512, 1) k_sweep_range_lpr(RangeParams p) {
+    typedef typename Acc<XT>::T AT;
+    typedef Word<XT> W;
+    typedef typename W::T WT;
+    constexpr int NA = V / 2;  // partial sums of a lane
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    WT* sxp = (WT*)smem_raw;
+    const unsigned int sbase = (unsigned int)__cvta_generic_to_shared(smem_raw);
+    const int lo = blockIdx.x * p.rows, hi = min(p.n, lo + p.rows);
+    const int turn = __ldcg(p.state);
+    for (int i = threadIdx.x; i < hi - lo; i += blockDim.x) sxp[i] = W::kSent;
+    __syncthreads();
+    const int c0 = __ldg(p.part_chunk + blockIdx.x), c1 = __ldg(p.part_chunk + blockIdx.x + 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int rsub = lane >> 1, half = lane & 1;
+    const VT* __restrict__ ev = (const VT*)p.ell_val;
+    const VT* __restrict__ tv = (const VT*)p.tval;
+    XT* xp = (XT*)p.xpb[turn];
+    auto chunk = [&](int c) { return c < c1 ? __ldg(p.chunks + c) : make_int2(0, 0); };
+    int c = c0 + warp;
+    int2 ch = chunk(c), ch1 = chunk(c + nwarps);
+    RangeIdx ix;
+    ix.load(p, ch, rsub);
+    for (; c < c1; c += nwarps) {
+        const int2 ch2 = chunk(c + 2 * nwarps);
+        RangeIdx ix1;
+        const int r = ch.x + rsub;
+        const bool act = rsub < ch.y;
+        AT acc[NA];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) acc[i] = AT(0);
+        AT diag = AT(1);
+        int t0 = 0, tl = 0;
+        if (act) {
+            if (half == 0) acc[0] = ld_rhs<AT>(p.b, p.b32, (long)ix.gr * p.ldb);
+            t0 = __ldg(p.tptr + r);
+            tl = __ldg(p.tptr + r + 1) - 1 - t0;
+            diag = (AT)__ldg((const XT*)p.dinv + r);
+        }
+        // slot k = 2 i + half of the row is this lane's i-th and goes to its partial sum i % NA
+        for (int ib = 0; 2 * ib < p.w; ib += NS) {
+            DepSlots<XT, AT, NS> slab;
+            slab.clear(sbase);
+#pragma unroll
+            for (int j = 0; j < NS; ++j) {
+                const int k = 2 * (ib + j) + half;
+                if (act && k < p.w) {
+                    const long s = (long)k * p.ld + r;
+                    range_set(slab, j, sbase, __ldg(p.ell_col + s), ldv<VT, AT>(ev + s));
+                }
+            }
+            if (ib == 0) ix1.load(p, ch1, rsub);
+            slab.wait(xp, p.status, p.budget);
+#pragma unroll
+            for (int j = 0; j < NS; ++j) {
+                if (2 * (ib + j) >= p.w) break;  // the same for every lane
+                acc[j % NA] = fma(-slab.v[j], (AT)W::val(slab.raw[j]), acc[j % NA]);
+            }
+        }
+        if (p.w == 0) ix1.load(p, ch1, rsub);
+        const int tmax = __reduce_max_sync(kFull, tl);
+        for (int tb = 0; tb < tmax; tb += V) {  // V tail entries of a row at a time
+            DepBatchP<XT, AT, NA> tail;
+            tail.clear();
+#pragma unroll
+            for (int j = 0; j < NA; ++j) {
+                const int t = tb + 2 * j + half;
+                if (t < tl) range_set(tail, j, sbase, __ldg(p.tcol + t0 + t), ldv<VT, AT>(tv + t0 + t));
+            }
+            tail.poll(xp);
+            tail.wait(xp, p.status, p.budget);
+#pragma unroll
+            for (int j = 0; j < NA; ++j)
+                if ((tail.valid >> j) & 1u) acc[j] = fma(-tail.v[j], (AT)W::val(tail.raw[j]), acc[j]);
+        }
+#pragma unroll
+        for (int h = NA / 2; h >= 1; h >>= 1)
+#pragma unroll
+            for (int i = 0; i < h; ++i) acc[i] += acc[i + h];
+        const AT xr = (acc[0] + __shfl_xor_sync(kFull, acc[0], 1)) * diag;
+        if (act && half == 0) {
+            if (r != p.skip_row) {
+                WT wv = sizeof(XT) == 8 ? (WT)__double_as_longlong((double)(XT)xr) : (WT)__float_as_uint((float)(XT)xr);
+                if (wv == W::kSent) wv = sizeof(XT) == 8 ? (WT)0x7FF8000000000000ull : (WT)0x7FC00000u;
+                *(volatile WT*)(sxp + (ix.id - lo)) = wv;
+                publish_x(xp + r, (XT)xr);
+            }
+            if (ix.sr >= 0) st_sol(p.x, p.x32, (long)ix.sr * p.ldx, xr);
+        }
+        ch = ch1;
+        ch1 = ch2;
+        ix = ix1;
+    }
+    WT* nxp = (WT*)p.xpb[turn ^ 1];
     for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) nxp[i] = W::kSent;
     if (threadIdx.x == 0 && atomicAdd(p.state + 1, 1) == (int)gridDim.x - 1) {
         p.state[1] = 0;
@@ -1529,15 +1651,19 @@ const void* part_kernel(int w) {
 
 namespace {
 template <typename VT, typename XT>
-const void* range_kernel(int w) {
+const void* range_kernel(int w, int v) {
+    if (v == 2) return (const void*)k_sweep_range_lpr<VT, XT, 2, 4>;
+    if (v == 4) return w <= 8 ? (const void*)k_sweep_range_lpr<VT, XT, 4, 4> : (const void*)k_sweep_range_lpr<VT, XT, 4, 8>;
+    if (v == 8) return w <= 8 ? (const void*)k_sweep_range_lpr<VT, XT, 8, 4> : (const void*)k_sweep_range_lpr<VT, XT, 8, 8>;
     return w <= 3   ? (const void*)k_sweep_range<VT, XT, 3>
            : w <= 4 ? (const void*)k_sweep_range<VT, XT, 4>
                     : (const void*)k_sweep_range<VT, XT, 8>;
 }
-const void* range_kernel(const hec_matrix* T) {
-    return T->vdt == HEC_F64 ? range_kernel<double, double>(T->w)
-           : T->vdt == HEC_F32 ? range_kernel<float, float>(T->w)
-                               : range_kernel<__nv_bfloat16, float>(T->w);
+// v: lanes per row of the global kernel whose sums are reproduced
+const void* range_kernel(const hec_matrix* T, int v) {
+    return T->vdt == HEC_F64 ? range_kernel<double, double>(T->w, v)
+           : T->vdt == HEC_F32 ? range_kernel<float, float>(T->w, v)
+                               : range_kernel<__nv_bfloat16, float>(T->w, v);
 }
 constexpr size_t kRangeSmem = 227 * 1024;  // shared solution of one block
 }  // namespace
@@ -1584,7 +1710,7 @@ hec_status sweep(const sptrsv_plan* pl, int nrhs, const double* b, int ldb, cons
             default: return dispatch_part<__nv_bfloat16, float>(pl, pp, s);
         }
     }
-    if (pl->range && pl->use_range && nrhs == 1 && pl->lpr1 == 1) {
+    if (pl->range && pl->use_range && nrhs == 1) {
         const hec_range_data* R = pl->range;
         RangeParams rp;
         rp.n = T->n;
@@ -1617,7 +1743,7 @@ hec_status sweep(const sptrsv_plan* pl, int nrhs, const double* b, int ldb, cons
         void* args[] = {&rp};
         void* tok = nullptr;
         profile_begin(s, &tok);
-        HEC_CUDA(cudaLaunchCooperativeKernel(range_kernel(T), dim3(R->nparts), dim3(R->threads), args,
+        HEC_CUDA(cudaLaunchCooperativeKernel(range_kernel(T, R->virt), dim3(R->nparts), dim3(R->threads), args,
                                              (size_t)R->rows * work_size(T->vdt), s));
         profile_end(s, tok);
         count_launch();
@@ -2034,10 +2160,10 @@ __device__ __forceinline__ int range_bound(const int* __restrict__ iperm, int a,
     }
     return a;
 }
-// (part q, level l) at q * nlev + l: its chunks of at most 32 rows, counted (chunks == NULL, into pos;
+// (part q, level l) at q * nlev + l: its chunks of at most rpw rows, counted (chunks == NULL, into pos;
 // nseg counts the nonempty ones, most[l] the most of a part) or written from pos
-__global__ void k_range_chunks(int n, int nlev, int nparts, int rows, int uplo, const int* __restrict__ iperm,
-                               const int* __restrict__ level_ptr, int* pos, int2* chunks, int* part_chunk,
+__global__ void k_range_chunks(int n, int nlev, int nparts, int rows, int rpw, int uplo,
+                               const int* __restrict__ iperm, const int* __restrict__ level_ptr, int* pos, int2* chunks, int* part_chunk,
                                int* most, unsigned long long* nseg) {
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= (long)nparts * nlev) return;
@@ -2046,7 +2172,7 @@ __global__ void k_range_chunks(int n, int nlev, int nparts, int rows, int uplo, 
     const int lo = q * rows, hi = min(n, lo + rows);  // original rows of the part
     const int r0 = range_bound(iperm, a, b, uplo ? hi : lo, uplo), r1 = range_bound(iperm, r0, b, uplo ? lo : hi, uplo);
     if (!chunks) {
-        const int cnt = (r1 - r0 + 31) / 32;
+        const int cnt = (r1 - r0 + rpw - 1) / rpw;
         pos[k] = cnt;
         if (cnt) {
             atomicAdd(nseg, 1ull);
@@ -2057,14 +2183,15 @@ __global__ void k_range_chunks(int n, int nlev, int nparts, int rows, int uplo, 
     int c = pos[k];
     if (l == 0) part_chunk[q] = c;
     if (k == (long)nparts * nlev - 1) part_chunk[nparts] = pos[k + 1];
-    for (int r = r0; r < r1; r += 32, ++c) chunks[c] = make_int2(r, min(32, r1 - r));
+    for (int r = r0; r < r1; r += rpw, ++c) chunks[c] = make_int2(r, min(rpw, r1 - r));
 }
 // estimated time of both schedules, summed over the levels, in units of 10 ns: a level takes the latency of
 // its hand-off or, when longer, the chunks of the block that has the most of them (ranges) or of an SM's
 // share (global).  cost[0] ranges, cost[1] global.
-__global__ void k_range_cost(int nlev, int sms, const int* __restrict__ level_ptr, const int* __restrict__ most,
+__global__ void k_range_cost(int nlev, int sms, int lanes, const int* __restrict__ level_ptr, const int* __restrict__ most,
                              unsigned long long* cost) {
-    constexpr int kHop = 45, kChunk = 12, kGlobalHop = 85, kGlobalChunk = 16;
+    const int kHop = lanes == 1 ? 45 : 85, kChunk = lanes == 1 ? 12 : 20, kGlobalHop = lanes == 1 ? 85 : 125,
+              kGlobalChunk = lanes == 1 ? 16 : 60;
     unsigned a = 0, b = 0;
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlev; l += gridDim.x * blockDim.x) {
         a += max(kHop, kChunk * most[l]);
@@ -2079,9 +2206,9 @@ __global__ void k_range_cost(int nlev, int sms, const int* __restrict__ level_pt
 }
 }  // namespace
 
-// The range schedule of a plan, when it pays and fits: a lane per row, the solution in the shared memory
+// The range schedule of a plan, when it pays and fits: the solution in the shared memory
 // of at most one block an SM, levels not so many that the (part, level) table outgrows the factor, at
-// most 60 % of the entries in another range (they would still meet in L2), and an estimated time at
+// most 80 % of the entries in another range (they would still meet in L2), and an estimated time at
 // least 15 % below the global schedule's (k_range_cost: a range whose level is many chunks is bound by
 // its one SM; its constants are fits to the times below).
 //   Parts: kRangeLevelRows rows of an average level each.  More parts cross more boundaries on the
@@ -2092,13 +2219,18 @@ __global__ void k_range_cost(int nlev, int sms, const int* __restrict__ level_pt
 // 31 x 37 x 29 161 / 80 (130 / 62), 50^3 245 / 129 (191 / 102), 64^3 323 / 172 (244 / 136), 100^3 548 / 359
 // (423 / 290), 128^3 723 / 486 (542 / 413), 160^3 937 / 726 (684 / 580); 576 Schwarz boxes of 128^3
 // 201 / 162 (177 / 116).  Where the estimate keeps the global one: 64 boxes 239 / 357 (193 / 270), FP32
-// 200^3 (921 / 926), random rows of six entries 248 / 390.
+// 200^3 (921 / 926), random rows of six entries 248 / 390.  More than four slots, global / range: ILU(1)
+// of the 7-point matrix 40^3 431 / 297 (307 / 210), 64^3 726 / 467 (588 / 331), 100^3 1178 / 1009.
+//   Long rows: two lanes each, 10 rows of an average level a part (20 rows: 64^3 1569 us).  27-point ILU(0)
+// 16^3 237 / 182 (158 / 109), 33 x 31 x 40 671 / 432 (585 / 329), 64^3 1161 / 1049 (1017 / 744), its ILUT
+// 64^3 1585 / 1129 (1237 / 770); ILU(2) of the 7-point matrix 64^3 1711 / 1328 (1249 / 867).
 hec_status build_range(sptrsv_plan* p) {
-    constexpr int kRangeLevelRows = 43;
+    const int kRangeLevelRows = p->lpr1 > 1 ? 10 : 43;
     const hec_matrix* T = p->T;
     const hec_levels* lv = p->lv;
     const int n = T->n, nlev = lv->nlev, sms = num_sms();
-    if (n == 0 || p->lpr1 != 1 || sms == 0) return HEC_OK;
+    const int virt = p->lpr1;
+    if (n == 0 || sms == 0 || (virt > 1 && T->w > 3 * virt)) return HEC_OK;
     const size_t ws = work_size(T->vdt);
     const long avg = (n + nlev - 1) / nlev;
     long need = (long)((ws * (size_t)n + kRangeSmem - 1) / kRangeSmem);
@@ -2106,6 +2238,9 @@ hec_status build_range(sptrsv_plan* p) {
     parts = std::max(1L, std::min(parts, (long)n));
     if (parts > sms || parts * nlev > 4L * n + 1024) return HEC_OK;
     hec_range_data* R = new hec_range_data();
+    R->virt = virt;
+    R->lanes = virt > 1 ? 2 : 1;
+    const int rpw = 32 / R->lanes;
     R->rows = (int)((n + parts - 1) / parts);
     R->nparts = (n + R->rows - 1) / R->rows;
     int *pos = nullptr, *most = nullptr;
@@ -2123,12 +2258,12 @@ hec_status build_range(sptrsv_plan* p) {
     };
     const long tbl = (long)R->nparts * nlev;
     if ((size_t)R->rows * ws > kRangeSmem ||
-        cudaFuncSetAttribute(range_kernel(T), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRangeSmem) != cudaSuccess) {
+        cudaFuncSetAttribute(range_kernel(T, virt), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRangeSmem) != cudaSuccess) {
         cudaGetLastError();
         free_range(R);
         return HEC_OK;
     }
-    R->cap_chunks = (int)std::min((long)n, tbl + n / 32);
+    R->cap_chunks = (int)std::min((long)n, tbl + n / rpw);
     if ((st = dalloc(&pos, (size_t)tbl + 1)) || (st = dalloc(&most, (size_t)nlev)) || (st = dalloc(&counts, 4)) || (st = dalloc(&R->chunks, (size_t)R->cap_chunks)) ||
         (st = dalloc(&R->part_chunk, (size_t)R->nparts + 1)) || (st = dalloc(&R->ell_col, (size_t)T->w * T->ld)) ||
         (st = dalloc(&R->tcol, (size_t)T->tail_nnz)) || (st = dmalloc(&R->xpb[0], ws * (size_t)n + 16)) ||
@@ -2138,11 +2273,11 @@ hec_status build_range(sptrsv_plan* p) {
         cudaMemsetAsync(most, 0, sizeof(int) * (size_t)nlev, s) != cudaSuccess)
         return done(cuda_error(cudaGetLastError(), "memset"));
     const int g = (int)((tbl + 127) / 128);
-    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, lv->uplo, lv->iperm, lv->level_ptr, pos, nullptr, nullptr,
+    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, pos, nullptr, nullptr,
                                      most, counts);
-    k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, lv->level_ptr, most, counts + 2);
+    k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, R->lanes, lv->level_ptr, most, counts + 2);
     if ((st = exclusive_scan_i32(pos, pos, (int)tbl, true, s))) return done(st);
-    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, lv->uplo, lv->iperm, lv->level_ptr, pos, R->chunks,
+    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, pos, R->chunks,
                                      R->part_chunk, most, counts);
     k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, T->ell_col, T->tptr, T->tcol, lv->iperm,
                                                      R->ell_col, R->tcol, counts + 1);
@@ -2159,10 +2294,13 @@ hec_status build_range(sptrsv_plan* p) {
     // 409 / 506, 1000 x 1000 1187 / 1488, 64^3 172 / 195, 100^3 392 / 359, 128^3 543 / 486)
     const long long nnz_bound = (long long)T->w * n + T->tail_nnz;
     const int seg_rows = n / (int)std::max(1ull, h[0]);
-    R->threads = seg_rows >= 40 && n >= 500000 ? 1024 : 512;
+    R->threads = R->lanes == 1 && T->w <= 4 && seg_rows >= 40 && avg >= 2000 ? 1024 : 512;
     const long long entries = nnz_bound - n;  // off-diagonals and padding
-    if ((long long)h[1] * 10 > entries * 6 || h[2] * 100 > h[3] * 85 ||
-        max_coop_blocks(range_kernel(T), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
+    // rows of more than four slots are not loaded a chunk ahead: a factor too large to stay in L2 then shows the
+    // latency of its loads (27-point ILU(0) on 100^3: 2116 us against 2086 for the global kernel)
+    const bool streams = (R->lanes > 1 || T->w > 4) && (double)T->w * n * (4 + (T->vdt == HEC_BF16 ? 2 : ws)) > 75e6;
+    if ((long long)h[1] * 10 > entries * 8 || h[2] * (streams ? 150 : 100) > h[3] * 85 ||
+        max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
         free_range(R);
         R = nullptr;
     }
@@ -2410,7 +2548,7 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
         }
     }
     if (st == HEC_OK && nrhs == 1 && p->range) {  // the range schedule (its launch shape is its own)
-        const TuneChoice c{bc.threads, bc.blocks, saved.lpr1, 0, 1};
+        const TuneChoice c{bc.threads, bc.blocks, bc.lpr1, 0, 1};
         apply_choice(p, c, nullptr);
         float ms = 0.f;
         st = time_it(&ms);

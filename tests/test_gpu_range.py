@@ -28,7 +28,12 @@ FACTORS = {  # name: (matrix, fill level, slab width)
     "box": (lambda: _box(40, 33, 27), 0, -1),
     "box_tail": (lambda: _box(19, 23, 17), 0, 1),                  # so long a tail that the default is two lanes a row
     "slim_tail": (lambda: _box(3, 3, 300), 0, 2),                  # a tail entry in some rows
-    "box_wide": (lambda: _box(19, 23, 17), 1, 6),                  # more slots than the kernel holds in registers
+    "box_wide": (lambda: _box(19, 23, 17), 1, 6),                  # eight slots a wait
+    "box_fill2": (lambda: _box(19, 23, 17), 2, -1),                # long rows: four partial sums, two lanes a row
+    "27pt": (lambda: synth.stencil27_jitter(21, seed=3), 0, -1),   # eight partial sums
+    "27pt_one_range": (lambda: synth.stencil27_jitter(9, seed=3), 0, 13),
+    "27pt_tail": (lambda: synth.stencil27_jitter(21, seed=3), 0, 6),   # two partial sums and a long tail
+    "27pt_w17": (lambda: synth.stencil27_jitter(12, seed=3), 1, 17),   # two waits a row, and a tail
     "box_pad": (lambda: _box(19, 23, 17), 0, 9),                   # slots that every row leaves empty
     "random": (lambda: synth.random_sparse(3000, 0.002, 4), 0, -1),
     "large": (lambda: _box(101, 97, 83), 0, -1),                   # 813,151 rows
