@@ -11,10 +11,14 @@
 // group's warps in turn; every warp takes its rows in increasing order, so the smallest unfinished
 // row can always proceed.  A row is tens of microseconds of work for one warp (a few for each
 // pivot), so the time is (rows / rows that can work at once): dealt one by one over all warps, only
-// W consecutive rows are in flight, one plane of a 100^3 grid, whose wavefront keeps 33 of the
-// 9,728 warps busy.  Groups put a dozen planes in flight, and a run held by a group holds back no row
+// W consecutive rows are in flight, half a plane of a 100^3 grid, whose wavefront keeps a few dozen of
+// the 4,864 warps busy.  Groups put a dozen planes in flight, and a run held by a group holds back no row
 // (each waits for the row before it anyway), while its warps work on the earlier pivots of the rows
-// ahead.  ILUT(10, 1e-3) of the 27-point stencil on 100^3 / 64^3 and of the 7-point matrix on 100^3:
+// ahead.  With enough rows at work the FP64 unit is the bound (16 SM-cycles a warp instruction): per row
+// about 25 divisions and 40 ranked candidates, so the ranking compares magnitudes as integers and the
+// division takes five FP64 instructions (div_by).  27-point 100^3 / 7-point 100^3: 45.2 / 37.7 ms with
+// FP64 compares and __ddiv_rn, 28.5 / 26.6 with integer compares, 22.0 / 23.2 with both.
+//   The groups, before that.  ILUT(10, 1e-3) of the 27-point stencil on 100^3 / 64^3 and of the 7-point matrix on 100^3:
 // row by row 167.6 / 45.1 / 189.0 ms, groups of 8 warps 45.2 / 17.2 / 37.7 (1 warp 100 / 39.7 / 110,
 // 4 warps 61.4 / 22.2 / 56.2, 16 warps 54.4 / 20.0 / 43.0, 32 warps 147 / 41.5 / 153).  Where there
 // are too few runs to give every group one, the groups grow (31 x 33 x 29: 4.9 / 5.2 ms).
@@ -53,6 +57,7 @@ struct IlutParams {
     int* llen;     // [n]
     int* ucol;     // [n * (p + 1)], diagonal first
     double* uval;
+    double* urcp;  // [n] reciprocals of the pivots
     int* ulen;     // [n], 0 until the row is published
     int* status;
     long long budget;
@@ -69,6 +74,22 @@ __device__ __forceinline__ int ld_acquire_flag(const int* p) {
 }
 __device__ __forceinline__ int ldcg_i(const int* p) { return __ldcg(p); }
 __device__ __forceinline__ double ldcg_d(const double* p) { return __ldcg(p); }
+
+// a / b for a pivot b whose reciprocal y = RN(1 / b) is kept with its row: Markstein's corrected quotient
+// (P. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990; IA-64
+// and Elementary Functions, 2000).  q1 = q0 + y (a - b q0) is within one ulp of a / b, and with y correctly
+// rounded q1 + y (a - b q1) rounds to RN(a / b), as long as no step leaves the normal range: the
+// exponents are checked, and anything else takes the division.  Five FP64 instructions.
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+    const int ea = (int)(((unsigned long long)__double_as_longlong(a) >> 52) & 0x7ff);
+    const int eb = (int)(((unsigned long long)__double_as_longlong(b) >> 52) & 0x7ff);
+    const int eq = ea - eb + 1023;
+    // a, b, 1 / b and the quotient well inside the normal range, and the residuals (about a / 2^53) too
+    if (ea < 120 || ea > 1900 || eb < 120 || eb > 1900 || eq < 120 || eq > 1900) return __ddiv_rn(a, b);
+    const double q0 = __dmul_rn(a, y);
+    const double q1 = __fma_rn(__fma_rn(-b, q0, a), y, q0);
+    return __fma_rn(__fma_rn(-b, q1, a), y, q1);
+}
 
 // position of the first entry with column >= c in cols[lo, hi)
 __device__ __forceinline__ int lower_bound(const int* cols, int lo, int hi, int c) {
@@ -95,12 +116,19 @@ __device__ __forceinline__ void ilut_publish(const IlutParams& P, int i, int lan
     __syncwarp();
 }
 
+// magnitude of a value as a word that compares like it (a NaN above everything)
+__device__ __forceinline__ unsigned long long mag(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
 // One strict part of a finished row, list positions [b0, b1): the entries with w != 0 and
-// |w| >= tau are the candidates; the p largest magnitudes are kept (ties to the smaller column)
+// |w| >= tau (least, as a word) are the candidates; the p largest magnitudes are kept (ties to the smaller column)
 // and written to out_col / out_val in column order.  The candidates are first compacted, in
 // column order, into the warp's spare buffer; up to 64 of them are ranked with shuffles (two per
-// lane), more by a scan of the compacted list.  Returns the number kept.
-__device__ __forceinline__ int ilut_select(const int* col, const double* val, int b0, int b1, double tau, int p,
+// lane), more by a scan of the compacted list.  Returns the number kept.  Magnitudes are compared
+// as integers: an FP64 compare occupies the SM's FP64 unit for 16 cycles, and four for each
+// candidate were half of the kernel's FP64 instructions.
+__device__ __forceinline__ int ilut_select(const int* col, const double* val, int b0, int b1, unsigned long long least, int p,
                                            int lane, int* scol, double* sval, int* out_col, double* out_val) {
     const unsigned lt = (1u << lane) - 1u;
     int m = 0;
@@ -108,8 +136,8 @@ __device__ __forceinline__ int ilut_select(const int* col, const double* val, in
         const int b = bb + lane;
         bool c = false;
         if (b < b1) {
-            const double v = val[b];
-            c = v != 0.0 && !(fabs(v) < tau);
+            const unsigned long long v = mag(val[b]);
+            c = v != 0ull && v >= least;
         }
         const unsigned cm = __ballot_sync(kAll, c);
         if (c) {
@@ -123,12 +151,14 @@ __device__ __forceinline__ int ilut_select(const int* col, const double* val, in
     int kept = 0;
     if (m <= 64) {
         const bool h0 = lane < m, h1 = lane + 32 < m;
-        const double a0 = h0 ? fabs(sval[lane]) : 0.0, a1 = h1 ? fabs(sval[lane + 32]) : 0.0;
+        const unsigned long long a0 = h0 ? mag(sval[lane]) : 0ull, a1 = h1 ? mag(sval[lane + 32]) : 0ull;
         int r0 = 0, r1 = 0;  // candidates ahead of this lane's two (larger, or equal with a smaller column)
-        for (int t = 0; t < m; ++t) {
-            const double at = __shfl_sync(kAll, t < 32 ? a0 : a1, t & 31);
-            r0 += (at > a0 || (at == a0 && t < lane)) ? 1 : 0;
-            r1 += (at > a1 || (at == a1 && t < lane + 32)) ? 1 : 0;
+        if (m > p) {
+            for (int t = 0; t < m; ++t) {
+                const unsigned long long at = __shfl_sync(kAll, t < 32 ? a0 : a1, t & 31);
+                r0 += (t < lane ? at >= a0 : at > a0) ? 1 : 0;
+                r1 += (t < lane + 32 ? at >= a1 : at > a1) ? 1 : 0;
+            }
         }
         const bool k0 = h0 && r0 < p, k1 = h1 && r1 < p;
         const unsigned m0 = __ballot_sync(kAll, k0), m1 = __ballot_sync(kAll, k1);
@@ -143,11 +173,11 @@ __device__ __forceinline__ int ilut_select(const int* col, const double* val, in
             const int e = eb + lane;
             bool k = false;
             if (e < m) {
-                const double ae = fabs(sval[e]);
+                const unsigned long long ae = mag(sval[e]);
                 int rank = 0;
                 for (int t = 0; t < m && rank < p; ++t) {
-                    const double at = fabs(sval[t]);
-                    rank += (at > ae || (at == ae && t < e)) ? 1 : 0;
+                    const unsigned long long at = mag(sval[t]);
+                    rank += (t < e ? at >= ae : at > ae) ? 1 : 0;
                 }
                 k = rank < p;
             }
@@ -166,6 +196,7 @@ __device__ __forceinline__ void ilut_fail(const IlutParams& P, int i, int lane, 
         record(P.status, code);
         P.ucol[(long)i * (P.p + 1)] = i;
         P.uval[(long)i * (P.p + 1)] = 1.0;
+        P.urcp[i] = 1.0;
         P.llen[i] = 0;
     }
     ilut_publish(P, i, lane, 1);
@@ -208,13 +239,15 @@ __global__ void __launch_bounds__(256) k_ilut(IlutParams P) {
         }
         __syncwarp();
         // tau = tol * ||a_i||_2, the squares summed in row order
-        double tau = 0.0;
-        if (lane == 0) {
-            double nrm = 0.0;
-            for (int e = 0; e < len; ++e) nrm = __dadd_rn(nrm, __dmul_rn(val[e], val[e]));
-            tau = __dmul_rn(P.tol, __dsqrt_rn(nrm));
+        double nrm = 0.0;
+        for (int eb = 0; eb < len; eb += 32) {  // 32 squares with one instruction, then the sum in order
+            const double v = eb + lane < len ? val[eb + lane] : 0.0;
+            const double sq = __dmul_rn(v, v);
+            const int m = min(32, len - eb);
+            for (int e = 0; e < m; ++e) nrm = __dadd_rn(nrm, __shfl_sync(kAll, sq, e));
         }
-        tau = __shfl_sync(kAll, tau, 0);
+        const double tau = __dmul_rn(P.tol, __dsqrt_rn(nrm));
+        const unsigned long long least = isnan(tau) ? 0ull : mag(tau);  // a NaN tau drops nothing
         // a structural diagonal slot when the row has none
         {
             const int dpos = lower_bound(col, 0, len, i);
@@ -250,13 +283,14 @@ __global__ void __launch_bounds__(256) k_ilut(IlutParams P) {
             // U row k's first 32 entries in one batch of loads; u_kk is its first entry
             int j0 = 0;
             double u0 = 0.0;
+            const double y = ldcg_d(P.urcp + k);
             if (lane < ul) {
                 j0 = ldcg_i(P.ucol + (long)k * up + lane);
                 u0 = ldcg_d(P.uval + (long)k * up + lane);
             }
-            const double wk = __ddiv_rn(val[pos], __shfl_sync(kAll, u0, 0));
+            const double wk = div_by(val[pos], __shfl_sync(kAll, u0, 0), y);
             __syncwarp();
-            if (fabs(wk) < tau) {  // dropped multiplier
+            if (mag(wk) < least) {  // dropped multiplier
                 if (lane == 0) val[pos] = 0.0;
                 __syncwarp();
                 continue;
@@ -314,14 +348,15 @@ __global__ void __launch_bounds__(256) k_ilut(IlutParams P) {
         if (wd == 0.0) { ilut_fail(P, i, lane, HEC_ERR_ZERO_PIVOT); continue; }
         int* scol = wc + (cur ^ 1) * cap;
         double* sval = wv + (cur ^ 1) * cap;
-        const int nu = ilut_select(col, val, dp + 1, len, tau, P.p, lane, scol, sval, P.ucol + (long)i * up + 1,
+        const int nu = ilut_select(col, val, dp + 1, len, least, P.p, lane, scol, sval, P.ucol + (long)i * up + 1,
                                    P.uval + (long)i * up + 1);
         if (lane == 0) {
             P.ucol[(long)i * up] = i;
             P.uval[(long)i * up] = wd;
+            P.urcp[i] = __drcp_rn(wd);
         }
         ilut_publish(P, i, lane, nu + 1);
-        const int nl = ilut_select(col, val, 0, dp, tau, P.p, lane, scol, sval, P.lcol + (long)i * P.p,
+        const int nl = ilut_select(col, val, 0, dp, least, P.p, lane, scol, sval, P.lcol + (long)i * P.p,
                                    P.lval + (long)i * P.p);
         if (lane == 0) P.llen[i] = nl;
     }
@@ -389,10 +424,10 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
     hec_csr *L = new hec_csr(), *U = new hec_csr();
     int *lcol = nullptr, *llen = nullptr, *ucol = nullptr, *ulen = nullptr, *status = nullptr, *lrl = nullptr,
         *url = nullptr, *runs = nullptr;
-    double *lval = nullptr, *uval = nullptr;
+    double *lval = nullptr, *uval = nullptr, *urcp = nullptr;
     auto cleanup = [&]() {
         dfree(lcol); dfree(llen); dfree(ucol); dfree(ulen); dfree(status); dfree(lrl);
-        dfree(url); dfree(runs); dfree(lval); dfree(uval);
+        dfree(url); dfree(runs); dfree(lval); dfree(uval); dfree(urcp);
     };
     auto fail = [&](hec_status e) {
         cleanup();
@@ -403,7 +438,7 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
     hec_status st = HEC_OK;
     const size_t ln = (size_t)n * p + 1, un = (size_t)n * (p + 1) + 1;
     if ((st = dalloc(&lcol, ln)) || (st = dalloc(&lval, ln)) || (st = dalloc(&llen, (size_t)n + 1)) ||
-        (st = dalloc(&ucol, un)) || (st = dalloc(&uval, un)) || (st = dalloc(&ulen, (size_t)n + 1)) ||
+        (st = dalloc(&ucol, un)) || (st = dalloc(&uval, un)) || (st = dalloc(&urcp, (size_t)n)) || (st = dalloc(&ulen, (size_t)n + 1)) ||
         (st = dalloc(&status, 1)) || (st = dalloc(&lrl, (size_t)n + 1)) || (st = dalloc(&url, (size_t)n + 1)) ||
         (st = dalloc(&L->rowptr, (size_t)n + 1)) || (st = dalloc(&U->rowptr, (size_t)n + 1)))
         return fail(st);
@@ -414,7 +449,7 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
     if (n > 0) {
         IlutParams P;
         P.n = n; P.p = p; P.tol = tol; P.rp = rowptr; P.ci = col; P.v = val;
-        P.lcol = lcol; P.lval = lval; P.llen = llen; P.ucol = ucol; P.uval = uval; P.ulen = ulen;
+        P.lcol = lcol; P.lval = lval; P.llen = llen; P.ucol = ucol; P.uval = uval; P.urcp = urcp; P.ulen = ulen;
         P.status = status;
         // the runs (lrl and url hold the flags and their prefix until the row lengths take them)
         const int gr = (n + 255) / 256;

@@ -78,6 +78,20 @@ ILUT = {
 }
 
 
+@pytest.mark.parametrize("scale", [1e-307, 1e-160, 1e-20, 1e150, 1e300])
+@pytest.mark.parametrize("p", [2, 40])
+def test_ilut_over_the_exponent_range_bitwise(p, scale):
+    """Quotients of the elimination: rows scaled over the range of FP64 (every third row by `scale`), so that some
+    pivots, values and quotients leave the range of the corrected reciprocal."""
+    A = synth.random_sparse(400, 0.02, 11)
+    row = np.repeat(np.arange(400), np.diff(A[0]))
+    A = (A[0], A[1], np.where(row % 3 == 0, A[2] * scale, A[2]))
+    from paper_1606_00541_gb300 import hec
+    for got, ref in zip(hec.ilut_factor(*dev(A), p=p, tol=1e-4), oracle.ilut(A, p, 1e-4)):
+        for x, y in zip(host(got), ref):
+            assert np.array_equal(x, y)
+
+
 @pytest.mark.parametrize("case", list(ILUT))
 def test_ilut_by_run_shape_bitwise(case):
     from paper_1606_00541_gb300 import hec
