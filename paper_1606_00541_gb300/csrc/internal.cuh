@@ -146,6 +146,7 @@ struct sptrsv_plan {
     const hec_levels* lv = nullptr;
     int max_nrhs = 1;
     int threads = 256, blocks = 0;
+    bool shaped = false;       // threads or blocks were asked for, or tuned
     long long wait_cycles = 2000000000LL;
     int skip_row = -1;         // fault injection: row never published (tests only)
     int backoff_ns = 0;        // sleep between dependency polls

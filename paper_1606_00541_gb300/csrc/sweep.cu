@@ -1489,10 +1489,16 @@ hec_status launch_sweep_vec(const sptrsv_plan* pl, SweepParams& sp, cudaStream_t
 template <typename VT, typename XT, int LPR>
 hec_status launch_sweep_lpr(const sptrsv_plan* pl, SweepParams& sp, cudaStream_t s) {
     const void* k = (const void*)k_sweep_lpr<VT, XT, LPR, 3, 2>;
-    const int threads = pl->threads;
+    // Unless the plan was given a shape: 16 warps an SM in blocks of 64 threads where 4 or 8 lanes share a
+    // row.  A level of long rows is a few chunks an SM, and more warps only add polls: L+U apply of the
+    // 27-point ILU(0), 8 lanes, 100^3 / 64^3: 256 threads and as many blocks as fit 2076 / 1160 us, 64 x 8
+    // 1838 / 1065, 128 x 4 1866 / 1089, 256 x 2 1933 / 1098; ILUT-like 4 lanes 3062 / 1738 against 2900 / 1688.
+    const bool def = !pl->shaped && LPR >= 4;
+    const int threads = def ? 64 : pl->threads;
     int per_sm = occupancy(k, threads);
     if (per_sm <= 0) return set_error(HEC_ERR_CUDA, "sweep kernel cannot be resident");
-    if (pl->blocks > 0) per_sm = std::min(per_sm, pl->blocks);
+    if (def) per_sm = std::min(per_sm, 8);
+    else if (pl->blocks > 0) per_sm = std::min(per_sm, pl->blocks);
     constexpr int idx = LPR == 2 ? 1 : LPR == 4 ? 2 : 3;
     if (!pl->chunks[idx]) return set_error(HEC_ERR_INVALID_ARG, "sweep: no chunk table for the plan's lanes per row");
     sp.chunks = pl->chunks[idx];
@@ -2336,6 +2342,7 @@ HEC_API hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* l
     p->lv = lv;
     p->max_nrhs = max_nrhs;
     if (tune) {
+        p->shaped = tune->block_threads || tune->blocks_per_sm;
         if (tune->block_threads) p->threads = tune->block_threads;
         if (tune->blocks_per_sm) p->blocks = tune->blocks_per_sm;
         if (tune->wait_cycles) p->wait_cycles = tune->wait_cycles;
@@ -2477,6 +2484,7 @@ void apply_choice(sptrsv_plan* p, const TuneChoice& c, hec_tune* out) {
     p->lpr1 = c.lpr1;
     p->use_part = c.use_part;
     p->use_range = c.use_range;
+    p->shaped = true;
     if (out) {
         *out = hec_tune{};
         out->block_threads = c.threads;
@@ -2515,6 +2523,7 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
+    const bool was_shaped = p->shaped;
     const TuneChoice saved{p->threads, p->blocks, p->lpr1, p->use_part, p->use_range};
     // one warm-up and three timed sweeps of the plan as it is set
     auto time_it = [&](float* ms) -> hec_status {
@@ -2565,7 +2574,7 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
     cudaEventDestroy(e1);
     dfree(b);
     dfree(x);
-    if (st) { apply_choice(p, saved, nullptr); return st; }
+    if (st) { apply_choice(p, saved, nullptr); p->shaped = was_shaped; return st; }
     apply_choice(p, bc, out);
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
