@@ -465,7 +465,8 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
         count_launch();
         P.runs = runs;
         P.nruns = nruns;
-        P.budget = 4000000000LL;  // about two seconds of SM cycles per wait
+        // about ten seconds of SM cycles per wait: a group waits for the wavefront to cross the planes in flight
+        P.budget = 20000000000LL;
         const void* k = (const void*)k_ilut;
         int h = 0, cap = 0;
         // a larger working list (fewer warps per block) only when a row's fill outgrew the last one

@@ -1108,8 +1108,8 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_part(PartParams p) {
 // word s of the range's shared solution, the level-ordered row for a row of another range, whose word
 // is polled in global memory (level order keeps a chunk's words in a few sectors).
 // Every row adds its entries in the order of k_sweep, so results are the same bit for bit.
-//   What bounds it is the latency of a level, as in the other sweeps: about 0.5 us where k_sweep takes 1
-// (its producers and consumers meet in L2).  Index loads run a chunk ahead of the row's loads, which
+//   What bounds it is the latency of a level, as in the other sweeps: 0.3 to 0.6 us where k_sweep takes
+// 0.65 to 0.9 (its producers and consumers meet in L2).  Index loads run a chunk ahead of the row's loads, which
 // for FP32 work run a chunk ahead of its wait.
 //   Both word buffers and the flag that says which one this sweep polls live on the device: the block
 // that finishes last turns the flag, so no fill launch is needed and a captured graph can be replayed.
@@ -2305,7 +2305,11 @@ hec_status build_range(sptrsv_plan* p) {
     // rows of more than four slots are not loaded a chunk ahead: a factor too large to stay in L2 then shows the
     // latency of its loads (27-point ILU(0) on 100^3: 2116 us against 2086 for the global kernel)
     const bool streams = (R->lanes > 1 || T->w > 4) && (double)T->w * n * (4 + (T->vdt == HEC_BF16 ? 2 : ws)) > 75e6;
-    if ((long long)h[1] * 10 > entries * 8 || h[2] * (streams ? 150 : 100) > h[3] * 85 ||
+    // the last range waits from the start of the sweep for the chain to reach it, where a warp of the global
+    // kernel only waits for the chunks in flight before its own: its wait must stay well inside the budget
+    // (four times the estimated sweep at 2.1 GHz)
+    const bool slow = (double)h[2] * 10.0 * 2.1 * 4.0 > (double)p->wait_cycles;
+    if (slow || (long long)h[1] * 10 > entries * 8 || h[2] * (streams ? 150 : 100) > h[3] * 85 ||
         max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
         free_range(R);
         R = nullptr;
@@ -2459,7 +2463,7 @@ HEC_API hec_status sptrsv_upper(const sptrsv_plan* p, int nrhs, const double* b,
 // tuned once per process.
 namespace {
 struct TuneKey {
-    int n, w, nlev, vdt, kp, parted;
+    int n, w, nlev, vdt, kp, parted;  // parted: 1 a partition, 2 the range schedule given
     long long tail;
     bool operator==(const TuneKey& o) const {
         return n == o.n && w == o.w && nlev == o.nlev && vdt == o.vdt && kp == o.kp && parted == o.parted &&
@@ -2503,7 +2507,7 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
     int kp = 1;
     while (kp < nrhs) kp <<= 1;
     const int parted = (nrhs == 1 && p->part) ? 1 : 0;
-    TuneKey key{T->n, T->w, p->lv->nlev, (int)T->vdt, kp, parted, T->tail_nnz};
+    TuneKey key{T->n, T->w, p->lv->nlev, (int)T->vdt, kp, parted + (nrhs == 1 && p->range ? 2 : 0), T->tail_nnz};
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_tune_cache.find(key);

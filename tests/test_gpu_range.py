@@ -79,6 +79,23 @@ def test_range_is_the_default_and_needs_one_launch():
     assert launches == [1, 2]  # the global kernel has a fill before it
 
 
+def test_short_wait_budget_keeps_the_global_schedule():
+    """58 levels are estimated at 26 us, 219,240 cycles with the factor of four: a smaller budget, and the plan sweeps
+    with the global kernel (two launches), whose waits are shorter."""
+    from paper_1606_00541_gb300 import hec
+    T = hec.ilu_factor(*dev(_box(20, 20, 20)), k=0)[0].tensors()
+    lv = hec.sptrsv_analyze(T[0], T[1], 0)
+    H = hec.hec_from_csr(*T, levels=lv)
+    b = torch.ones(8000, dtype=torch.float64, device="cuda")
+    launches = []
+    for budget in (0, 300_000, 200_000):
+        plan = hec.sptrsv_plan_create(H, lv, wait_cycles=budget)
+        before = hec.launch_count()
+        hec.sptrsv_lower(plan, b)
+        launches.append(hec.launch_count() - before)
+    assert launches == [1, 1, 2]
+
+
 def test_range_in_a_captured_graph():
     """Replays poll the word buffer the replay before them reset: an odd number of sweeps a graph."""
     from paper_1606_00541_gb300 import hec
