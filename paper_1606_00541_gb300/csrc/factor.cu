@@ -91,6 +91,21 @@ __global__ void __launch_bounds__(kIluWarps * 32) k_ilu_numeric(int n, const int
         bool bad = false;
         for (int p = 0; p < dpos; ++p) {
             const int k = rc[p];
+            // Everything of row k but its values is known before it is finished: its range, the column of
+            // this lane's first entry and that column's place in row i.  After the flag one load of values
+            // remains, the pivot and the lane's entry together.
+            const int dk = __ldg(dg + k), ek = __ldg(rp + k + 1);
+            int q = dk + 1 + lane;
+            int pos = len;
+            auto place = [&]() {
+                pos = len;
+                if (q < ek) {
+                    const int j = __ldg(col + q);
+                    const int at = lower_bound_i(rc, p + 1, len, j);
+                    if (at < len && rc[at] == j) pos = at;
+                }
+            };
+            place();
             // every lane acquires row k (bounded), so its reads of row k are ordered after the release
             bool ready = ld_acquire_i32(done + k) != 0;
             if (!__all_sync(full, ready)) {
@@ -105,8 +120,8 @@ __global__ void __launch_bounds__(kIluWarps * 32) k_ilu_numeric(int n, const int
                 }
             }
             if (bad) break;
-            const int dk = __ldg(dg + k), ek = __ldg(rp + k + 1);
             const double piv = lu[dk];
+            double u = pos < len ? lu[q] : 0.0;
             if (piv == 0.0) {
                 if (lane == 0) record(status, HEC_ERR_ZERO_PIVOT);
                 continue;
@@ -115,12 +130,12 @@ __global__ void __launch_bounds__(kIluWarps * 32) k_ilu_numeric(int n, const int
             __syncwarp();
             if (lane == 0) rv[p] = lik;
             for (int qb = dk + 1; qb < ek; qb += 32) {
-                const int q = qb + lane;
-                if (q < ek) {
-                    const int j = __ldg(col + q);
-                    const int pos = lower_bound_i(rc, p + 1, len, j);
-                    if (pos < len && rc[pos] == j) rv[pos] = fma(-lik, lu[q], rv[pos]);
+                if (qb > dk + 1) {
+                    q = qb + lane;
+                    place();
+                    u = pos < len ? lu[q] : 0.0;
                 }
+                if (pos < len) rv[pos] = fma(-lik, u, rv[pos]);
             }
             __syncwarp();
         }
