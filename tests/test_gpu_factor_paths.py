@@ -99,3 +99,19 @@ def test_ilut_by_run_shape_bitwise(case):
     for got, ref in zip(hec.ilut_factor(*dev(A), p=6, tol=1e-3), oracle.ilut(A, 6, 1e-3)):
         for x, y in zip(host(got), ref):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("scale", [1e-300, 1e-20, 1e150])
+def test_ilu0_over_the_exponent_range(scale):
+    """Warp-per-row elimination of rows scaled over the range of FP64 (every third row by `scale`): the quotients are
+    those of the division, so the factors stay within the rounding of a fused update."""
+    from paper_1606_00541_gb300 import hec
+    A = _banded(600, range(-6, 7))
+    row = np.repeat(np.arange(600), np.diff(A[0]))
+    A = (A[0], A[1], np.where(row % 3 == 0, A[2] * scale, A[2]))
+    for got, ref in zip(hec.ilu_factor(*dev(A), k=0), oracle.ilu0(A)):
+        rp, ci, v = host(got)
+        assert np.array_equal(rp, ref[0]) and np.array_equal(ci, ref[1]) and np.isfinite(v).all()
+        r = np.repeat(np.arange(600), np.diff(rp))
+        big = np.maximum.reduceat(np.abs(ref[2]), rp[:-1])[r]  # row by row: the rows differ in scale
+        assert np.all(np.abs(v - ref[2]) <= 1e-12 * big)
