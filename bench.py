@@ -612,7 +612,7 @@ class Schedule:
             s.partition(self.part, self.nparts, threads=part_threads(self.m))
 
     def kernel(self):
-        return {"global": "k_sweep<float,float,1,4>", "part": "k_sweep_part<float,float,4>"}[self.kind]
+        return {"global": "k_sweep<float,float,1,4>", "part": "k_sweep_part<float,float,3>"}[self.kind]
 
     def describe(self):
         if self.kind == "part":
