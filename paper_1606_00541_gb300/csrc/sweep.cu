@@ -15,6 +15,7 @@
 // Multiple right-hand sides: lane = (row of the warp's chunk, right-hand side), with the
 // right-hand sides of a row interleaved, so one slab entry serves up to 16 solves.
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <string>
 #include <unordered_map>
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(256) k_sweep(SweepParams p) {
 // same bits; the fixed pairing makes the result deterministic (it differs from the one-lane
 // kernel only in summation order).
 template <typename VT, typename XT, int LPR, int SPL, int TB>
-__global__ void __launch_bounds__(256) k_sweep_lpr(SweepParams p) {
+__global__ void __launch_bounds__(256, LPR == 2 && sizeof(VT) == 2 ? 6 : 0) k_sweep_lpr(SweepParams p) {
     typedef typename Acc<XT>::T AT;
     constexpr int NS = SPL + TB;
     const int lane = threadIdx.x & 31;
@@ -1427,17 +1428,43 @@ int occupancy(const void* k, int threads) {
     return nb;
 }
 
+// Block size and resident blocks an SM of a global sweep: what the plan was given or tuned to, else by the
+// width of the levels.  A warp that is resident and not at the wavefront only polls, and with scattered
+// words (ILUT, coloured and random orderings: a sector each) the polls alone can keep L2 busy.  An SM that
+// has c chunks of an average level needs the warps of that level and of the next few: 10 a chunk, in eights.
+// Levels so wide that the sweep is bound by bandwidth get all that fit.
+// L+U apply, all that fit / 8 warps an SM, 100^3: ILUT of the 27-point matrix (c = 0.3), one lane a row, FP32
+// 10740 / 3565 us, FP64 5181 / 4502, four right-hand sides FP32 5616 / 4008; its ILU(0), one lane, FP32 5455 / 4855; ILU(0) /
+// ILU(1) of the 7-point matrix (0.7 / 0.3), FP64 553 / 531 and FP32 1058 / 860; 1000 x 1000 grid, FP64 2828 / 2591.
+// 8 / 16 / 24 warps / all: 7-point 128^3 (1.1) FP32 611 / 542 / 543 / 557, 160^3 (1.8) 966 / 732 / 689 / 703.
+// A random ordering of the 7-point 64^3 (3.0), 8 / 16 warps / all: FP64 76.9 / 73.5 / 77.5.  Eight colours of the 27-point
+// 100^3 (26): FP32 348 / 196 / 128.
+//   With 4 or 8 lanes a row at least 16 warps, in blocks of 64 threads: the 27-point ILU(0), 8 lanes, 100^3 (2.4) /
+// 64^3: 256 threads and as many blocks as fit 2076 / 1160 us, 64 x 8 1838 / 1065, 128 x 4 1866 / 1089, 256 x 2
+// 1933 / 1098; its eight colours (200): as many as fit 333 us, 64 x 8 708.
+struct SweepShape {
+    int threads, per_sm;
+};
+SweepShape sweep_shape(const sptrsv_plan* pl, const void* k, int nchunks, bool many_lanes) {
+    if (pl->shaped) {
+        const int fit = occupancy(k, pl->threads);
+        return {pl->threads, pl->blocks > 0 ? std::min(fit, pl->blocks) : fit};
+    }
+    const double c = nchunks / ((double)std::max(1, pl->lv->nlev) * std::max(1, num_sms()));
+    const int eights = (int)std::max(1.0, std::min(8.0, std::ceil(1.25 * c)));  // at most 64 warps an SM
+    if (many_lanes && c <= 4.0) return {64, std::min(8, occupancy(k, 64))};
+    return {256, std::min(eights, occupancy(k, 256))};
+}
+
 template <typename VT, typename XT, int KP, int WMAX>
 hec_status launch_sweep(const sptrsv_plan* pl, SweepParams& sp, cudaStream_t s) {
     const void* k = (const void*)k_sweep<VT, XT, KP, WMAX>;
-    const int threads = pl->threads;
-    int per_sm = occupancy(k, threads);
-    if (per_sm <= 0) return set_error(HEC_ERR_CUDA, "sweep kernel cannot be resident");
-    if (pl->blocks > 0) per_sm = std::min(per_sm, pl->blocks);
     constexpr int kp_idx = KP == 1 ? 0 : KP == 2 ? 1 : KP == 4 ? 2 : KP == 8 ? 3 : 4;
     if (!pl->chunks[kp_idx]) return set_error(HEC_ERR_INVALID_ARG, "sweep: nrhs above the plan's max_nrhs");
     sp.chunks = pl->chunks[kp_idx];
     sp.nchunks = pl->nchunks[kp_idx];
+    const auto [threads, per_sm] = sweep_shape(pl, k, sp.nchunks, false);
+    if (per_sm <= 0) return set_error(HEC_ERR_CUDA, "sweep kernel cannot be resident");
     long nchunks = sp.nchunks;
     long want = (nchunks + threads / 32 - 1) / (threads / 32);
     int blocks = (int)std::max(1L, std::min((long)per_sm * num_sms(), want));
@@ -1460,14 +1487,12 @@ hec_status launch_sweep(const sptrsv_plan* pl, SweepParams& sp, cudaStream_t s) 
 template <typename VT, typename XT, int LPR, int G, int WMAX>
 hec_status launch_sweep_vec(const sptrsv_plan* pl, SweepParams& sp, cudaStream_t s) {
     const void* k = (const void*)k_sweep_vec<VT, XT, LPR, G, WMAX>;
-    const int threads = pl->threads;
-    int per_sm = occupancy(k, threads);
-    if (per_sm <= 0) return set_error(HEC_ERR_CUDA, "sweep kernel cannot be resident");
-    if (pl->blocks > 0) per_sm = std::min(per_sm, pl->blocks);
     constexpr int idx = LPR == 1 ? 0 : LPR == 2 ? 1 : LPR == 4 ? 2 : LPR == 8 ? 3 : 4;
     if (!pl->chunks[idx]) return set_error(HEC_ERR_INVALID_ARG, "sweep: nrhs above the plan's max_nrhs");
     sp.chunks = pl->chunks[idx];
     sp.nchunks = pl->nchunks[idx];
+    const auto [threads, per_sm] = sweep_shape(pl, k, sp.nchunks, false);
+    if (per_sm <= 0) return set_error(HEC_ERR_CUDA, "sweep kernel cannot be resident");
     const long want = ((long)sp.nchunks + threads / 32 - 1) / (threads / 32);
     const int blocks = (int)std::max(1L, std::min((long)per_sm * num_sms(), want));
     const long count = (long)sp.n * LPR * G;
@@ -1489,20 +1514,12 @@ hec_status launch_sweep_vec(const sptrsv_plan* pl, SweepParams& sp, cudaStream_t
 template <typename VT, typename XT, int LPR>
 hec_status launch_sweep_lpr(const sptrsv_plan* pl, SweepParams& sp, cudaStream_t s) {
     const void* k = (const void*)k_sweep_lpr<VT, XT, LPR, 3, 2>;
-    // Unless the plan was given a shape: 16 warps an SM in blocks of 64 threads where 4 or 8 lanes share a
-    // row.  A level of long rows is a few chunks an SM, and more warps only add polls: L+U apply of the
-    // 27-point ILU(0), 8 lanes, 100^3 / 64^3: 256 threads and as many blocks as fit 2076 / 1160 us, 64 x 8
-    // 1838 / 1065, 128 x 4 1866 / 1089, 256 x 2 1933 / 1098; ILUT-like 4 lanes 3062 / 1738 against 2900 / 1688.
-    const bool def = !pl->shaped && LPR >= 4;
-    const int threads = def ? 64 : pl->threads;
-    int per_sm = occupancy(k, threads);
-    if (per_sm <= 0) return set_error(HEC_ERR_CUDA, "sweep kernel cannot be resident");
-    if (def) per_sm = std::min(per_sm, 8);
-    else if (pl->blocks > 0) per_sm = std::min(per_sm, pl->blocks);
     constexpr int idx = LPR == 2 ? 1 : LPR == 4 ? 2 : 3;
     if (!pl->chunks[idx]) return set_error(HEC_ERR_INVALID_ARG, "sweep: no chunk table for the plan's lanes per row");
     sp.chunks = pl->chunks[idx];
     sp.nchunks = pl->nchunks[idx];
+    const auto [threads, per_sm] = sweep_shape(pl, k, sp.nchunks, LPR >= 4);
+    if (per_sm <= 0) return set_error(HEC_ERR_CUDA, "sweep kernel cannot be resident");
     const long want = ((long)sp.nchunks + threads / 32 - 1) / (threads / 32);
     const int blocks = (int)std::max(1L, std::min((long)per_sm * num_sms(), want));
     const long count = sp.n;

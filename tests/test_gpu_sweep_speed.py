@@ -1,0 +1,70 @@
+"""Sweeps against one another in time, where a wait's polls decide it: a schedule or value type that moves fewer words
+must not be the slower one.  The fastest of several passes on each side; margins are far from both figures measured."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1606_00541_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(A):
+    return [torch.as_tensor(np.ascontiguousarray(a), device="cuda") for a in A]
+
+
+def shuffled(A, seed):
+    """The matrix with its rows and columns in a random order."""
+    rp, ci, v = A
+    n = len(rp) - 1
+    new = synth._rng(seed).permutation(n)
+    r, c = new[np.repeat(np.arange(n), np.diff(rp))], new[ci]
+    order = np.lexsort((c, r))
+    out = np.zeros(n + 1, np.int32)
+    out[1:] = np.cumsum(np.bincount(r, minlength=n))
+    return out, c[order].astype(np.int32), v[order]
+
+
+def fastest(calls, reps=12):
+    """Of each call: the least time of `reps` passes, taken in turn."""
+    best = [float("inf")] * len(calls)
+    for f in calls:
+        f()
+    for _ in range(reps):
+        for i, f in enumerate(calls):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            f()
+            b.record()
+            b.synchronize()
+            best[i] = min(best[i], a.elapsed_time(b) * 1e3)
+    return best
+
+
+def apply_of(hec, L, U, n, nrhs=1, **kw):
+    s = hec.IluSolver(L, U, max_nrhs=nrhs, **kw)
+    b = torch.ones((n, nrhs) if nrhs > 1 else n, dtype=torch.float64, device="cuda")
+    z = torch.empty_like(b)
+    return s, lambda: s.apply(b, z)
+
+
+def test_one_lane_a_row_of_scattered_words():
+    """ILUT(10, 1e-3) of the 27-point 64^3, one lane a row: FP32 takes 0.7 times as long as FP64 (1.5 / 2.3 ms); with all the
+    warps that fit, each with eight words a lane outstanding, 1.5 times."""
+    from paper_1606_00541_gb300 import hec
+    n = 64 ** 3
+    L, U = [h.tensors() for h in hec.ilut_factor(*dev(synth.stencil27_jitter(64, seed=1)), p=10, tol=1e-3)]
+    t64, t32 = fastest([apply_of(hec, L, U, n, vdt=vdt, lanes_per_row=1)[1] for vdt in ("f64", "f32")])
+    assert t32 <= 1.1 * t64, (t32, t64)
+
+
+@pytest.mark.parametrize("lanes", [4, 8])
+def test_wide_levels_get_all_warps(lanes):
+    """ILU(0) of a random ordering of the 7-point 100^3, levels of thousands of rows, several lanes a row: the plan's own shape
+    against 256 threads and as many blocks as fit (16 warps an SM: up to twice as long on such levels)."""
+    from paper_1606_00541_gb300 import hec
+    n = 100 ** 3
+    A = dev(shuffled(synth.poisson3d_7pt(100), 5))
+    L, U = [h.tensors() for h in hec.ilu_factor(*A, k=0)]
+    own, full = fastest([apply_of(hec, L, U, n, vdt="f32", lanes_per_row=lanes, **kw)[1] for kw in ({}, dict(block_threads=256))])
+    assert own <= 1.25 * full, (own, full)
