@@ -709,7 +709,20 @@ struct DepBatchP {
             where[k] = (unsigned int)cc;
         }
     }
+    // All words at once, as in warp_wait; eight FP64 words one by one: read together they do not fit the 64
+    // registers of a 1024-thread block (ILU(1) of the 7-point 100^3 in 76 parts, L+U apply at once / one by one:
+    // FP64 2640 / 1790 us, FP32, which fits, 940 / 1160).
     __device__ __forceinline__ void poll(const XT* xp) {
+        if constexpr (sizeof(WT) == 8 && NS > 4) {
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                if ((pend >> k) & 1u) {
+                    raw[k] = (local >> k) & 1u ? (WT)ld_shared_u64(where[k]) : W::load(xp + where[k]);
+                    if (raw[k] != W::kSent) pend &= ~(1u << k);
+                }
+            }
+            return;
+        }
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
             const bool here = (local >> k) & 1u, on = (pend >> k) & 1u;

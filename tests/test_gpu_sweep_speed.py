@@ -68,3 +68,19 @@ def test_wide_levels_get_all_warps(lanes):
     L, U = [h.tensors() for h in hec.ilu_factor(*A, k=0)]
     own, full = fastest([apply_of(hec, L, U, n, vdt="f32", lanes_per_row=lanes, **kw)[1] for kw in ({}, dict(block_threads=256))])
     assert own <= 1.25 * full, (own, full)
+
+
+def test_partitioned_fp64_of_six_slots():
+    """ILU(1) of the 7-point 100^3 in 76 parts.  FP64 takes about 1.9 times as long as FP32 (1790 / 940 us); with its eight
+    words polled at once, and spilled, 2.8 times."""
+    from paper_1606_00541_gb300 import hec
+    n = 100 ** 3
+    L, U = [h.tensors() for h in hec.ilu_factor(*dev(synth.poisson3d_7pt(100)), k=1)]
+    part = (torch.arange(n, device="cuda") * 76 // n).to(torch.int32)
+    calls = []
+    for vdt in ("f64", "f32"):
+        s, f = apply_of(hec, L, U, n, vdt=vdt)
+        s.partition(part, 76, threads=512)
+        calls.append(f)
+    t64, t32 = fastest(calls)
+    assert t64 <= 2.3 * t32, (t64, t32)
