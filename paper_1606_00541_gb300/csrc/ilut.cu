@@ -21,7 +21,9 @@
 //   The groups, before that.  ILUT(10, 1e-3) of the 27-point stencil on 100^3 / 64^3 and of the 7-point matrix on 100^3:
 // row by row 167.6 / 45.1 / 189.0 ms, groups of 8 warps 45.2 / 17.2 / 37.7 (1 warp 100 / 39.7 / 110,
 // 4 warps 61.4 / 22.2 / 56.2, 16 warps 54.4 / 20.0 / 43.0, 32 warps 147 / 41.5 / 153).  Where there
-// are too few runs to give every group one, the groups grow (31 x 33 x 29: 4.9 / 5.2 ms).
+// are too few runs to give every group one, the groups grow (31 x 33 x 29: 4.9 / 5.2 ms); a group is never larger than a
+// run of average length, since only as many of its warps have a row of a run (eight colours of the 27-point 64^3,
+// runs of one row: groups of 8 warps 36.8 ms, of one 8.3; red-black 7-point 100^3 201 / 33.1).
 //   A warp keeps its row as a sorted (column, value) list in shared memory; merging U row k is a
 // warp-parallel binary search plus a ballot-ranked insertion of the fill.  A finished row is
 // written into fixed slots (p strictly lower, 1 + p upper entries) and published with a release
@@ -468,7 +470,8 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
                           cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess))
                 return fail(cuda_error(cudaGetLastError(), "ilut_factor: memset"));
             P.cap = cap;
-            P.g = std::min(blocks * warps, std::max(kRunWarps, 2 * blocks * warps / std::max(1, nruns)));
+            P.g = std::max(kRunWarps, 2 * blocks * warps / std::max(1, nruns));
+            P.g = std::max(1, std::min({P.g, blocks * warps, n / std::max(1, nruns)}));
             void* args[] = {&P};
             if (cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(warps * 32), args, smem, s) != cudaSuccess)
                 return fail(cuda_error(cudaGetLastError(), "ilut_factor: launch"));
