@@ -68,7 +68,9 @@ struct IlutParams {
     const int* __restrict__ runs;  // [nruns + 1] first row of each run
     int nruns;
     int g;         // warps that share a run
+    int* made;     // [kMade * 8] rows published, counted in kMade words of 32 bytes each
 };
+constexpr int kMade = 64;
 
 __device__ __forceinline__ int ld_acquire_flag(const int* p) {
     int v;
@@ -97,10 +99,33 @@ namespace {
 __device__ __forceinline__ void ilut_publish(const IlutParams& P, int i, int lane, int nu1) {
     __syncwarp();
     if (lane == 0) {
+        atomicAdd(P.made + 8 * (blockIdx.x % kMade), 1);
         __threadfence();
         st_release_i32(P.ulen + i, nu1);
     }
     __syncwarp();
+}
+
+// U row k's length, waited for; -1 when the wait gave up.  A wait can span every row of the runs in flight (half of
+// the matrix for one long chain), so its budget is for the time without any row published by anyone: when it
+// has run out, the wait goes on if the count of rows has moved since it last ran out.
+__device__ __forceinline__ int ilut_wait(const IlutParams& P, int k) {
+    int ul = ld_acquire_flag(P.ulen + k);
+    if (ul != 0) return ul;
+    long long t0 = clock64();
+    unsigned seen = 0u;  // rows published when the budget last ran out
+    for (unsigned it = 1; (ul = ld_acquire_flag(P.ulen + k)) == 0; ++it) {
+        if ((it & 63u) != 0u) continue;
+        if (ld_relaxed_u32(P.status) != 0u) return -1;
+        if (clock64() - t0 > P.budget) {
+            unsigned made = 0u;
+            for (int w = 0; w < kMade; ++w) made += ld_relaxed_u32(P.made + 8 * w);
+            if (made == seen) return -1;
+            seen = made;
+            t0 = clock64();
+        }
+    }
+    return ul;
 }
 
 // magnitude of a value as a word that compares like it (a NaN above everything)
@@ -254,17 +279,7 @@ __global__ void __launch_bounds__(256) k_ilut(IlutParams P) {
         for (int pos = 0; pos < len && col[pos] < i; ++pos) {
             const int k = col[pos];
             int ul = 0;
-            if (lane == 0) {
-                ul = ld_acquire_flag(P.ulen + k);
-                if (ul == 0) {
-                    const long long t0 = clock64();
-                    for (unsigned it = 1; (ul = ld_acquire_flag(P.ulen + k)) == 0; ++it)
-                        if ((it & 63u) == 0u && (clock64() - t0 > P.budget || ld_relaxed_u32(P.status) != 0u)) {
-                            ul = -1;
-                            break;
-                        }
-                }
-            }
+            if (lane == 0) ul = ilut_wait(P, k);
             ul = __shfl_sync(kAll, ul, 0);
             if (ul < 0) { failed = HEC_ERR_TIMEOUT; break; }
             // U row k's first 32 entries in one batch of loads; u_kk is its first entry
@@ -426,11 +441,11 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
     const size_t ln = (size_t)n * p + 1, un = (size_t)n * (p + 1) + 1;
     if ((st = dalloc(&lcol, ln)) || (st = dalloc(&lval, ln)) || (st = dalloc(&llen, (size_t)n + 1)) ||
         (st = dalloc(&ucol, un)) || (st = dalloc(&uval, un)) || (st = dalloc(&urcp, (size_t)n)) || (st = dalloc(&ulen, (size_t)n + 1)) ||
-        (st = dalloc(&status, 1)) || (st = dalloc(&lrl, (size_t)n + 1)) || (st = dalloc(&url, (size_t)n + 1)) ||
+        (st = dalloc(&status, 8 + 8 * kMade)) || (st = dalloc(&lrl, (size_t)n + 1)) || (st = dalloc(&url, (size_t)n + 1)) ||
         (st = dalloc(&L->rowptr, (size_t)n + 1)) || (st = dalloc(&U->rowptr, (size_t)n + 1)))
         return fail(st);
     if (cudaMemsetAsync(ulen, 0, sizeof(int) * ((size_t)n + 1), s) != cudaSuccess ||
-        cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess)
+        cudaMemsetAsync(status, 0, sizeof(int) * (8 + 8 * kMade), s) != cudaSuccess)
         return fail(cuda_error(cudaGetLastError(), "ilut_factor: memset"));
     L->n = U->n = n;
     if (n > 0) {
@@ -452,8 +467,8 @@ HEC_API hec_status ilut_factor(int n, const int* rowptr, const int* col, const d
         count_launch();
         P.runs = runs;
         P.nruns = nruns;
-        // about ten seconds of SM cycles per wait: a group waits for the wavefront to cross the planes in flight
-        P.budget = 20000000000LL;
+        P.budget = 4000000000LL;  // about two seconds of SM cycles without a row published
+        P.made = status + 8;
         const void* k = (const void*)k_ilut;
         int h = 0, cap = 0;
         // a larger working list (fewer warps per block) only when a row's fill outgrew the last one

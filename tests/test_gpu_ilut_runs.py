@@ -59,3 +59,27 @@ def test_coloured_factors_bitwise():
     for got, ref in zip(hec.ilut_factor(*dev(A), p=8, tol=1e-3), oracle.ilut(A, 8, 1e-3)):
         for x, y in zip(got.tensors(), ref):
             assert np.array_equal(x.cpu().numpy(), y)
+
+
+def test_one_chain_of_millions_of_rows():
+    """A band of seven diagonals: with half of the matrix in flight, the last warps wait 11 seconds for the rows before
+    theirs.  A wait gives up only when no row has been published for two.  The leading factors against the oracle's."""
+    from paper_1606_00541_gb300 import hec
+    n, lead = 5_000_000, 5000
+    cols = torch.arange(n, device="cuda")[:, None] + torch.arange(-3, 4, device="cuda")
+    inside = (cols >= 0) & (cols < n)
+    v = -torch.rand(n, 7, device="cuda", dtype=torch.float64, generator=torch.Generator(device="cuda").manual_seed(3))
+    v[:, 3] = 6.0
+    rp = torch.zeros(n + 1, dtype=torch.int32, device="cuda")
+    rp[1:] = inside.sum(1).cumsum(0)
+    A = rp, cols[inside].to(torch.int32), v[inside]
+    L, U = hec.ilut_factor(*A, p=3, tol=0.0)
+    first = inside[:lead] & (cols[:lead] < lead)
+    B = [np.concatenate([[0], first.sum(1).cumsum(0).cpu().numpy()]).astype(np.int32),
+         cols[:lead][first].cpu().numpy().astype(np.int32), v[:lead][first].cpu().numpy()]
+    rows = lead - 8  # the last rows of the block lack columns
+    for got, ref in zip((L, U), oracle.ilut(B, 3, 0.0)):
+        rp, ci, va = got.tensors()
+        k = int(ref[0][rows])
+        assert np.array_equal(rp[:rows + 1].cpu().numpy(), ref[0][:rows + 1])
+        assert np.array_equal(ci[:k].cpu().numpy(), ref[1][:k]) and np.array_equal(va[:k].cpu().numpy(), ref[2][:k])
