@@ -2159,14 +2159,16 @@ hec_status build_partition(sptrsv_plan* p, const int* part, int nparts, cudaStre
 }
 
 namespace {
-// the columns of slab and tail coded by where their words are (see RangeParams); *ncross: entries whose
-// row is in another range
-__global__ void k_range_cols(int n, int ld, int w, int rows, const int* __restrict__ ec, const int* __restrict__ tp,
-                             const int* __restrict__ tc, const int* __restrict__ iperm, int* oec, int* otc,
-                             unsigned long long* ncross) {
+// the columns of slab and tail coded by where their words are (see RangeParams); ncross[0]: entries whose
+// row is in another range, ncross[1]: the longest tail (without the diagonal) of each 32 rows, in waits of
+// `batch` entries, summed, ncross[2]: how many 32 rows have a tail
+__global__ void k_range_cols(int n, int ld, int w, int rows, int batch, const int* __restrict__ ec,
+                             const int* __restrict__ tp, const int* __restrict__ tc, const int* __restrict__ iperm, int* oec,
+                             int* otc, unsigned long long* ncross) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    int cross = 0;
+    int cross = 0, waits = 0;
     if (r < n) {
+        waits = (__ldg(tp + r + 1) - __ldg(tp + r) - 1 + batch - 1) / batch;
         const int q = __ldg(iperm + r) / rows;
         auto code = [&](int c) {
             const int j = __ldg(iperm + c);
@@ -2184,7 +2186,14 @@ __global__ void k_range_cols(int n, int ld, int w, int rows, const int* __restri
         for (int k = 0; k < w; ++k) oec[(long)k * ld + r] = -1;
     }
     cross = __reduce_add_sync(0xffffffffu, cross);
-    if ((threadIdx.x & 31) == 0 && cross) atomicAdd(ncross, (unsigned long long)cross);
+    waits = __reduce_max_sync(0xffffffffu, waits);
+    if ((threadIdx.x & 31) == 0) {
+        if (cross) atomicAdd(ncross, (unsigned long long)cross);
+        if (waits) {
+            atomicAdd(ncross + 1, (unsigned long long)waits);
+            atomicAdd(ncross + 2, 1ull);
+        }
+    }
 }
 // first row in [a, b) of a level whose original number, ascending (descending for an upper factor), has
 // reached v
@@ -2280,7 +2289,8 @@ hec_status build_range(sptrsv_plan* p) {
     R->rows = (int)((n + parts - 1) / parts);
     R->nparts = (n + R->rows - 1) / R->rows;
     int *pos = nullptr, *most = nullptr;
-    unsigned long long* counts = nullptr;  // nonempty (part, level) pairs; entries in another range; costs
+    // nonempty (part, level) pairs; entries in another range; waits for tails by 32 rows, and such 32 rows; costs
+    unsigned long long* counts = nullptr;
     hec_status st = HEC_OK;
     cudaStream_t s = 0;
     auto done = [&](hec_status e) {
@@ -2300,28 +2310,28 @@ hec_status build_range(sptrsv_plan* p) {
         return HEC_OK;
     }
     R->cap_chunks = (int)std::min((long)n, tbl + n / rpw);
-    if ((st = dalloc(&pos, (size_t)tbl + 1)) || (st = dalloc(&most, (size_t)nlev)) || (st = dalloc(&counts, 4)) || (st = dalloc(&R->chunks, (size_t)R->cap_chunks)) ||
+    if ((st = dalloc(&pos, (size_t)tbl + 1)) || (st = dalloc(&most, (size_t)nlev)) || (st = dalloc(&counts, 6)) || (st = dalloc(&R->chunks, (size_t)R->cap_chunks)) ||
         (st = dalloc(&R->part_chunk, (size_t)R->nparts + 1)) || (st = dalloc(&R->ell_col, (size_t)T->w * T->ld)) ||
         (st = dalloc(&R->tcol, (size_t)T->tail_nnz)) || (st = dmalloc(&R->xpb[0], ws * (size_t)n + 16)) ||
         (st = dmalloc(&R->xpb[1], ws * (size_t)n + 16)) || (st = dalloc(&R->state, 2)))
         return done(st);
-    if (cudaMemsetAsync(R->state, 0, 2 * sizeof(int), s) != cudaSuccess || cudaMemsetAsync(counts, 0, 4 * sizeof(*counts), s) != cudaSuccess ||
+    if (cudaMemsetAsync(R->state, 0, 2 * sizeof(int), s) != cudaSuccess || cudaMemsetAsync(counts, 0, 6 * sizeof(*counts), s) != cudaSuccess ||
         cudaMemsetAsync(most, 0, sizeof(int) * (size_t)nlev, s) != cudaSuccess)
         return done(cuda_error(cudaGetLastError(), "memset"));
     const int g = (int)((tbl + 127) / 128);
     k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, pos, nullptr, nullptr,
                                      most, counts);
-    k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, R->lanes, lv->level_ptr, most, counts + 2);
+    k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, R->lanes, lv->level_ptr, most, counts + 4);
     if ((st = exclusive_scan_i32(pos, pos, (int)tbl, true, s))) return done(st);
     k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, pos, R->chunks,
                                      R->part_chunk, most, counts);
-    k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, T->ell_col, T->tptr, T->tcol, lv->iperm,
-                                                     R->ell_col, R->tcol, counts + 1);
+    k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, R->lanes == 1 ? kTailBatch : virt, T->ell_col,
+                                                     T->tptr, T->tcol, lv->iperm, R->ell_col, R->tcol, counts + 1);
     const int fb = std::min(4096, (n + 255) / 256);  // the words of the first sweep; each sweep sets its successor's
     if (ws == 8) k_fill_sentinel<double><<<fb, 256, 0, s>>>((double*)R->xpb[0], n);
     else k_fill_sentinel<float><<<fb, 256, 0, s>>>((float*)R->xpb[0], n);
     count_launch(5);
-    unsigned long long h[4] = {0, 0, 0, 0};
+    unsigned long long h[6] = {};
     if (cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return done(cuda_error(cudaGetLastError(), "range schedule"));
@@ -2333,13 +2343,20 @@ hec_status build_range(sptrsv_plan* p) {
     R->threads = R->lanes == 1 && T->w <= 4 && seg_rows >= 40 && avg >= 2000 ? 1024 : 512;
     const long long entries = nnz_bound - n;  // off-diagonals and padding
     // rows of more than four slots are not loaded a chunk ahead: a factor too large to stay in L2 then shows the
-    // latency of its loads (27-point ILU(0) on 100^3: 2116 us against 2086 for the global kernel)
-    const bool streams = (R->lanes > 1 || T->w > 4) && (double)T->w * n * (4 + (T->vdt == HEC_BF16 ? 2 : ws)) > 75e6;
+    // latency of its loads (27-point ILU(0) on 100^3: 2116 us against 2086 for the global kernel, ILUT BF16 2100 / 1710)
+    const bool streams =
+        (R->lanes > 1 || T->w > 4) &&
+        (double)(R->lanes > 1 ? nnz_bound : (long long)T->w * n) * (4 + (T->vdt == HEC_BF16 ? 2 : ws)) > (R->lanes > 1 ? 65e6 : 75e6);
+    // rows with a tail wait once for each V entries of the chunk's longest (see the kernel), 0.35 us each beyond the
+    // first, where the global kernel takes 2 V entries together with the slab's; the chain runs through such rows
+    // (red-black 7-point 100^3, ILU(1) and ILUT, FP32, L+U apply with ranges / global: 1193 / 823, 1637 / 1288 us)
+    const double tail_waits = R->lanes > 1 ? (double)h[2] / (double)std::max(1ull, h[3]) : 0.0;
+    h[4] += (unsigned long long)(35.0 * std::max(0.0, tail_waits - 1.0) * nlev);
     // the last range waits from the start of the sweep for the chain to reach it, where a warp of the global
     // kernel only waits for the chunks in flight before its own: its wait must stay well inside the budget
     // (four times the estimated sweep at 2.1 GHz)
-    const bool slow = (double)h[2] * 10.0 * 2.1 * 4.0 > (double)p->wait_cycles;
-    if (slow || (long long)h[1] * 10 > entries * 8 || h[2] * (streams ? 150 : 100) > h[3] * 85 ||
+    const bool slow = (double)h[4] * 10.0 * 2.1 * 4.0 > (double)p->wait_cycles;
+    if (slow || (long long)h[1] * 10 > entries * 8 || h[4] * (streams ? 150 : 100) > h[5] * 85 ||
         max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
         free_range(R);
         R = nullptr;
