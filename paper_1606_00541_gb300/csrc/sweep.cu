@@ -2159,22 +2159,42 @@ hec_status build_partition(sptrsv_plan* p, const int* part, int nparts, cudaStre
 }
 
 namespace {
-// the columns of slab and tail coded by where their words are (see RangeParams); ncross[0]: entries whose
-// row is in another range, ncross[1]: the longest tail (without the diagonal) of each 32 rows, in waits of
-// `batch` entries, summed, ncross[2]: how many 32 rows have a tail
-__global__ void k_range_cols(int n, int ld, int w, int rows, int batch, const int* __restrict__ ec,
-                             const int* __restrict__ tp, const int* __restrict__ tc, const int* __restrict__ iperm, int* oec,
-                             int* otc, unsigned long long* ncross) {
+// what the choice needs to know of the columns: counts[0] += entries whose row is in another range, counts[1] +=
+// the longest tail (without the diagonal) of each 32 rows, in waits of `batch` entries, counts[2] += how many 32
+// rows have a tail
+__global__ void k_range_count(int n, int ld, int w, int rows, int batch, const int* __restrict__ ec,
+                              const int* __restrict__ tp, const int* __restrict__ tc, const int* __restrict__ iperm,
+                              unsigned long long* counts) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     int cross = 0, waits = 0;
     if (r < n) {
-        waits = (__ldg(tp + r + 1) - __ldg(tp + r) - 1 + batch - 1) / batch;
+        const int q = __ldg(iperm + r) / rows, t0 = __ldg(tp + r), t1 = __ldg(tp + r + 1) - 1;
+        waits = (t1 - t0 + batch - 1) / batch;
+        for (int k = 0; k < w; ++k) {
+            const int c = __ldg(ec + (long)k * ld + r);
+            cross += c >= 0 && __ldg(iperm + c) / rows != q;
+        }
+        for (int t = t0; t < t1; ++t) cross += __ldg(iperm + __ldg(tc + t)) / rows != q;
+    }
+    cross = __reduce_add_sync(0xffffffffu, cross);
+    waits = __reduce_max_sync(0xffffffffu, waits);
+    if ((threadIdx.x & 31) == 0) {
+        if (cross) atomicAdd(counts, (unsigned long long)cross);
+        if (waits) {
+            atomicAdd(counts + 1, (unsigned long long)waits);
+            atomicAdd(counts + 2, 1ull);
+        }
+    }
+}
+// the columns of slab and tail coded by where their words are (see RangeParams)
+__global__ void k_range_cols(int n, int ld, int w, int rows, const int* __restrict__ ec, const int* __restrict__ tp,
+                             const int* __restrict__ tc, const int* __restrict__ iperm, int* oec, int* otc) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < n) {
         const int q = __ldg(iperm + r) / rows;
         auto code = [&](int c) {
             const int j = __ldg(iperm + c);
-            if (j / rows == q) return -2 - (j - q * rows);
-            ++cross;
-            return c;
+            return j / rows == q ? -2 - (j - q * rows) : c;
         };
         for (int k = 0; k < w; ++k) {
             const long s = (long)k * ld + r;
@@ -2184,15 +2204,6 @@ __global__ void k_range_cols(int n, int ld, int w, int rows, int batch, const in
         for (int t = __ldg(tp + r); t < __ldg(tp + r + 1); ++t) otc[t] = code(__ldg(tc + t));
     } else if (r < ld) {
         for (int k = 0; k < w; ++k) oec[(long)k * ld + r] = -1;
-    }
-    cross = __reduce_add_sync(0xffffffffu, cross);
-    waits = __reduce_max_sync(0xffffffffu, waits);
-    if ((threadIdx.x & 31) == 0) {
-        if (cross) atomicAdd(ncross, (unsigned long long)cross);
-        if (waits) {
-            atomicAdd(ncross + 1, (unsigned long long)waits);
-            atomicAdd(ncross + 2, 1ull);
-        }
     }
 }
 // first row in [a, b) of a level whose original number, ascending (descending for an upper factor), has
@@ -2205,30 +2216,61 @@ __device__ __forceinline__ int range_bound(const int* __restrict__ iperm, int a,
     }
     return a;
 }
-// (part q, level l) at q * nlev + l: its chunks of at most rpw rows, counted (chunks == NULL, into pos;
-// nseg counts the nonempty ones, most[l] the most of a part) or written from pos
-__global__ void k_range_chunks(int n, int nlev, int nparts, int rows, int rpw, int uplo,
-                               const int* __restrict__ iperm, const int* __restrict__ level_ptr, int* pos, int2* chunks, int* part_chunk,
-                               int* most, unsigned long long* nseg) {
+// rows [r0, r1) of part q in level l
+__device__ __forceinline__ int2 range_rows(int q, int l, int n, int rows, int uplo, const int* __restrict__ iperm,
+                                           const int* __restrict__ level_ptr) {
+    const int b = __ldg(level_ptr + l + 1), lo = q * rows, hi = min(n, lo + rows);  // original rows of the part
+    const int r0 = range_bound(iperm, __ldg(level_ptr + l), b, uplo ? hi : lo, uplo);
+    return make_int2(r0, range_bound(iperm, r0, b, uplo ? lo : hi, uplo));
+}
+// chunks of at most rpw rows by (part, level): nseg counts the nonempty pairs, most[l] is the most of a part, total[q]
+// a part's
+__global__ void k_range_chunk_counts(int n, int nlev, int nparts, int rows, int rpw, int uplo, const int* __restrict__ iperm,
+                                     const int* __restrict__ level_ptr, int* most, int* total, unsigned long long* nseg) {
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= (long)nparts * nlev) return;
     const int q = (int)(k / nlev), l = (int)(k - (long)q * nlev);
-    const int a = __ldg(level_ptr + l), b = __ldg(level_ptr + l + 1);
-    const int lo = q * rows, hi = min(n, lo + rows);  // original rows of the part
-    const int r0 = range_bound(iperm, a, b, uplo ? hi : lo, uplo), r1 = range_bound(iperm, r0, b, uplo ? lo : hi, uplo);
-    if (!chunks) {
-        const int cnt = (r1 - r0 + rpw - 1) / rpw;
-        pos[k] = cnt;
-        if (cnt) {
-            atomicAdd(nseg, 1ull);
-            atomicMax(most + l, cnt);
-        }
-        return;
+    const int2 r = range_rows(q, l, n, rows, uplo, iperm, level_ptr);
+    const int cnt = (r.y - r.x + rpw - 1) / rpw;
+    if (!cnt) return;
+    atomicAdd(nseg, 1ull);
+    atomicMax(most + l, cnt);
+    atomicAdd(total + q, cnt);
+}
+// the chunk table, a block per part: the parts before it by their totals, its levels by a scan
+constexpr int kRangeTableThreads = 256;
+__global__ void __launch_bounds__(kRangeTableThreads) k_range_chunks(int n, int nlev, int nparts, int rows, int rpw, int uplo,
+                                                                     const int* __restrict__ iperm,
+                                                                     const int* __restrict__ level_ptr,
+                                                                     const int* __restrict__ total, int2* chunks, int* part_chunk) {
+    __shared__ int warp_sum[kRangeTableThreads / 32];
+    const int q = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int base = 0;
+    for (int i = 0; i < q; ++i) base += __ldg(total + i);
+    if (threadIdx.x == 0) {
+        part_chunk[q] = base;
+        if (q == nparts - 1) part_chunk[nparts] = base + __ldg(total + q);
     }
-    int c = pos[k];
-    if (l == 0) part_chunk[q] = c;
-    if (k == (long)nparts * nlev - 1) part_chunk[nparts] = pos[k + 1];
-    for (int r = r0; r < r1; r += rpw, ++c) chunks[c] = make_int2(r, min(rpw, r1 - r));
+    for (int l0 = 0; l0 < nlev; l0 += kRangeTableThreads) {
+        const int l = l0 + threadIdx.x;
+        const int2 r = l < nlev ? range_rows(q, l, n, rows, uplo, iperm, level_ptr) : make_int2(0, 0);
+        const int cnt = (r.y - r.x + rpw - 1) / rpw;
+        int x = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFull, x, o);
+            if (lane >= o) x += y;
+        }
+        __syncthreads();  // the sums of the step before have been read
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        int c = base + x - cnt;
+        for (int i = 0; i < kRangeTableThreads / 32; ++i) {
+            if (i < warp) c += warp_sum[i];
+            base += warp_sum[i];
+        }
+        for (int a = r.x; a < r.y; a += rpw, ++c) chunks[c] = make_int2(a, min(rpw, r.y - a));
+    }
 }
 // estimated time of both schedules, summed over the levels, in units of 10 ns: a level takes the latency of
 // its hand-off or, when longer, the chunks of the block that has the most of them (ranges) or of an SM's
@@ -2288,20 +2330,6 @@ hec_status build_range(sptrsv_plan* p) {
     const int rpw = 32 / R->lanes;
     R->rows = (int)((n + parts - 1) / parts);
     R->nparts = (n + R->rows - 1) / R->rows;
-    int *pos = nullptr, *most = nullptr;
-    // nonempty (part, level) pairs; entries in another range; waits for tails by 32 rows, and such 32 rows; costs
-    unsigned long long* counts = nullptr;
-    hec_status st = HEC_OK;
-    cudaStream_t s = 0;
-    auto done = [&](hec_status e) {
-        dfree(pos); dfree(most); dfree(counts);
-        if (e != HEC_OK) free_range(R);
-        if (e == HEC_ERR_OOM) {  // no room: the plan keeps the global schedule
-            clear_error();
-            return HEC_OK;
-        }
-        return e;
-    };
     const long tbl = (long)R->nparts * nlev;
     if ((size_t)R->rows * ws > kRangeSmem ||
         cudaFuncSetAttribute(range_kernel(T, virt), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRangeSmem) != cudaSuccess) {
@@ -2309,29 +2337,35 @@ hec_status build_range(sptrsv_plan* p) {
         free_range(R);
         return HEC_OK;
     }
-    R->cap_chunks = (int)std::min((long)n, tbl + n / rpw);
-    if ((st = dalloc(&pos, (size_t)tbl + 1)) || (st = dalloc(&most, (size_t)nlev)) || (st = dalloc(&counts, 6)) || (st = dalloc(&R->chunks, (size_t)R->cap_chunks)) ||
-        (st = dalloc(&R->part_chunk, (size_t)R->nparts + 1)) || (st = dalloc(&R->ell_col, (size_t)T->w * T->ld)) ||
-        (st = dalloc(&R->tcol, (size_t)T->tail_nnz)) || (st = dmalloc(&R->xpb[0], ws * (size_t)n + 16)) ||
-        (st = dmalloc(&R->xpb[1], ws * (size_t)n + 16)) || (st = dalloc(&R->state, 2)))
-        return done(st);
-    if (cudaMemsetAsync(R->state, 0, 2 * sizeof(int), s) != cudaSuccess || cudaMemsetAsync(counts, 0, 6 * sizeof(*counts), s) != cudaSuccess ||
-        cudaMemsetAsync(most, 0, sizeof(int) * (size_t)nlev, s) != cudaSuccess)
+    // The choice comes before any table of the size of the factor: counts of the chunks and a pass over the columns, in one
+    // block of memory.  counts: nonempty (part, level) pairs; entries in another range; waits for tails by 32 rows, and such
+    // 32 rows; costs
+    unsigned long long* counts = nullptr;
+    cudaStream_t s = 0;
+    auto done = [&](hec_status e) {
+        dfree(counts);
+        if (e != HEC_OK) free_range(R);
+        if (e == HEC_ERR_OOM) {  // no room: the plan keeps the global schedule
+            clear_error();
+            return HEC_OK;
+        }
+        return e;
+    };
+    constexpr int kCounts = 6;
+    const size_t scratch = kCounts * sizeof(*counts) + sizeof(int) * ((size_t)nlev + R->nparts);
+    hec_status st = dmalloc((void**)&counts, scratch);
+    if (st) return done(st);
+    int *most = (int*)(counts + kCounts), *total = most + nlev;
+    if (cudaMemsetAsync(counts, 0, scratch, s) != cudaSuccess)
         return done(cuda_error(cudaGetLastError(), "memset"));
     const int g = (int)((tbl + 127) / 128);
-    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, pos, nullptr, nullptr,
-                                     most, counts);
+    k_range_chunk_counts<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, most, total,
+                                           counts);
     k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, R->lanes, lv->level_ptr, most, counts + 4);
-    if ((st = exclusive_scan_i32(pos, pos, (int)tbl, true, s))) return done(st);
-    k_range_chunks<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, pos, R->chunks,
-                                     R->part_chunk, most, counts);
-    k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, R->lanes == 1 ? kTailBatch : virt, T->ell_col,
-                                                     T->tptr, T->tcol, lv->iperm, R->ell_col, R->tcol, counts + 1);
-    const int fb = std::min(4096, (n + 255) / 256);  // the words of the first sweep; each sweep sets its successor's
-    if (ws == 8) k_fill_sentinel<double><<<fb, 256, 0, s>>>((double*)R->xpb[0], n);
-    else k_fill_sentinel<float><<<fb, 256, 0, s>>>((float*)R->xpb[0], n);
-    count_launch(5);
-    unsigned long long h[6] = {};
+    k_range_count<<<(n + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, R->lanes == 1 ? kTailBatch : virt, T->ell_col, T->tptr,
+                                                  T->tcol, lv->iperm, counts + 1);
+    count_launch(3);
+    unsigned long long h[kCounts] = {};
     if (cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return done(cuda_error(cudaGetLastError(), "range schedule"));
@@ -2359,10 +2393,27 @@ hec_status build_range(sptrsv_plan* p) {
     if (slow || (long long)h[1] * 10 > entries * 8 || h[4] * (streams ? 150 : 100) > h[5] * 85 ||
         max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
         free_range(R);
-        R = nullptr;
+        return done(HEC_OK);
     }
+    R->cap_chunks = (int)std::min((long)n, tbl + n / rpw);
+    if ((st = dalloc(&R->chunks, (size_t)R->cap_chunks)) || (st = dalloc(&R->part_chunk, (size_t)R->nparts + 1)) ||
+        (st = dalloc(&R->ell_col, (size_t)T->w * T->ld)) || (st = dalloc(&R->tcol, (size_t)T->tail_nnz)) ||
+        (st = dmalloc(&R->xpb[0], ws * (size_t)n + 16)) || (st = dmalloc(&R->xpb[1], ws * (size_t)n + 16)) ||
+        (st = dalloc(&R->state, 2)))
+        return done(st);
+    if (cudaMemsetAsync(R->state, 0, 2 * sizeof(int), s) != cudaSuccess) return done(cuda_error(cudaGetLastError(), "memset"));
+    k_range_chunks<<<R->nparts, kRangeTableThreads, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr,
+                                                            total, R->chunks, R->part_chunk);
+    k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, T->ell_col, T->tptr, T->tcol, lv->iperm,
+                                                     R->ell_col, R->tcol);
+    const int fb = std::min(4096, (n + 255) / 256);  // the words of the first sweep; each sweep sets its successor's
+    if (ws == 8) k_fill_sentinel<double><<<fb, 256, 0, s>>>((double*)R->xpb[0], n);
+    else k_fill_sentinel<float><<<fb, 256, 0, s>>>((float*)R->xpb[0], n);
+    count_launch(3);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return done(cuda_error(e, "range schedule"));
     p->range = R;
-    return done(HEC_OK);
+    return done(HEC_OK);  // which waits for the device (dfree)
 }
 
 // resident blocks of the partitioned kernel for `smem` bytes of shared solution per block
