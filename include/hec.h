@@ -169,8 +169,11 @@ hec_status hec_matrix_destroy(hec_matrix* A);
 /* ---------------------------------------------------------------------------------------- */
 
 typedef struct {
-    int block_threads;      /* threads per block of the sweep kernel (0 = 256) */
-    int blocks_per_sm;      /* resident blocks per SM (0 = as many as fit) */
+    int block_threads;      /* threads per block of the global sweep kernels; 0 with blocks_per_sm 0: by the
+                               chunks an SM has of an average level (256, or 64 where 4 or 8 lanes share a
+                               row and levels are narrow); 0 with blocks_per_sm given: 256 */
+    int blocks_per_sm;      /* resident blocks per SM (0 = by the same rule, or as many as fit when
+                               block_threads is given) */
     long long wait_cycles;  /* SM cycles a dependency wait may spin before HEC_ERR_TIMEOUT
                                (0 = 2e9, about one second) */
     int debug_unpublished_row; /* fault injection for tests: a new (level-ordered) row whose
@@ -186,16 +189,27 @@ typedef struct {
                                dependencies in one wait and add their partial sums with an xor
                                butterfly (a different summation order from one lane). */
     int partitioned;        /* output of sptrsv_autotune: 1 when single-right-hand-side sweeps of
-                               the plan take its partition (sptrsv_plan_partition), 0 when the
-                               global schedule was faster or there is no partition; ignored as
+                               the plan take its partition (sptrsv_plan_partition), 0 when another
+                               schedule was faster or there is no partition; ignored as
                                an input */
+    int schedule;           /* HEC_SCHEDULE_*.  Input: AUTO (0) = the range schedule where it pays and no
+                               shape, lanes or backoff is given; GLOBAL = never the range schedule;
+                               RANGE = the range schedule where it pays, also with a shape and lanes
+                               given; PART = as AUTO (the partition itself is given with
+                               sptrsv_plan_partition).  Output of sptrsv_autotune: what sweeps of the
+                               tuned number of right-hand sides now run.  block_threads and blocks_per_sm then are
+                               the fastest shape of the global kernels, which RANGE and PART sweeps do not
+                               use, and lanes_per_row that of the global kernels, or with RANGE the lanes
+                               whose sums the ranges reproduce.  A plan created with the whole output runs the
+                               same schedule (with PART, once it is partitioned). */
 } hec_tune;
+enum { HEC_SCHEDULE_AUTO = 0, HEC_SCHEDULE_GLOBAL = 1, HEC_SCHEDULE_RANGE = 2, HEC_SCHEDULE_PART = 3 };
 
 /* A solve plan for one triangular factor: its HEC form and level analysis (both borrowed; they
  * must outlive the plan) plus the workspace for up to max_nrhs right-hand sides
  * (1 <= max_nrhs <= 16).  tune may be NULL for defaults.
- * A plan for one right-hand side with the default launch shape and lanes per row also gets, where it
- * pays and device memory allows, the range schedule: contiguous ranges of original rows, one resident
+ * A plan for one right-hand side (max_nrhs = 1) with the default launch shape and lanes per row, or with
+ * HEC_SCHEDULE_RANGE, also gets, where it pays and device memory allows, the range schedule: contiguous ranges of original rows, one resident
  * block each with its solution in shared memory, results as the global schedule's bit for bit.  It
  * keeps a copy of the factor's column indices and two n-entry solution buffers. */
 hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* lv, int max_nrhs,
@@ -247,7 +261,7 @@ int sptrsv_partition_capacity(const sptrsv_plan* p, int threads);
  * (sptrsv_plan_partition), the partitioned schedule against the best global one (a plan whose
  * global schedule wins keeps its partition unused; partitioning it again re-enables it).
  * Results are cached per (rows, slab width, tail entries, levels, value type, nrhs rounded up to
- * a power of two, partition given) for the life of the process.  Synchronizes `stream`.  The
+ * a power of two, partition given, range schedule present) for the life of the process.  Synchronizes `stream`.  The
  * point-to-point sweep has no per-level barriers, so the paper's level-merging threshold has no
  * counterpart. */
 hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void* stream);

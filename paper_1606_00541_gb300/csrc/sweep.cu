@@ -2317,7 +2317,7 @@ hec_status build_range(sptrsv_plan* p) {
     const hec_levels* lv = p->lv;
     const int n = T->n, nlev = lv->nlev, sms = num_sms();
     const int virt = p->lpr1;
-    if (n == 0 || sms == 0 || (virt > 1 && T->w > 3 * virt)) return HEC_OK;
+    if (n == 0 || sms == 0 || T->w > (virt > 1 ? 3 * virt : 8)) return HEC_OK;  // the slots the kernels take
     const size_t ws = work_size(T->vdt);
     const long avg = (n + nlev - 1) / nlev;
     long need = (long)((ws * (size_t)n + kRangeSmem - 1) / kRangeSmem);
@@ -2457,6 +2457,10 @@ HEC_API hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* l
         delete p;
         return set_error(HEC_ERR_INVALID_ARG, "sptrsv_plan_create: lanes_per_row must be 0, 1, 2, 4 or 8");
     }
+    if (tune && (tune->schedule < HEC_SCHEDULE_AUTO || tune->schedule > HEC_SCHEDULE_PART)) {
+        delete p;
+        return set_error(HEC_ERR_INVALID_ARG, "sptrsv_plan_create: schedule must be one of HEC_SCHEDULE_*");
+    }
     if (p->threads % 32 || p->threads < 32 || p->threads > 256) {
         delete p;
         return set_error(HEC_ERR_INVALID_ARG, "sptrsv_plan_create: block_threads must be a multiple of 32 in [32, 256]");
@@ -2470,7 +2474,9 @@ HEC_API hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* l
     if (st == HEC_OK) st = build_dinv(p);
     // a launch shape or lane layout asked for by the caller is that of the global kernels
     const bool shaped = tune && (tune->block_threads || tune->blocks_per_sm || tune->backoff_ns || tune->lanes_per_row);
-    if (st == HEC_OK && max_nrhs == 1 && !shaped) st = build_range(p);
+    const int schedule = tune ? tune->schedule : HEC_SCHEDULE_AUTO;
+    if (st == HEC_OK && max_nrhs == 1 && (schedule == HEC_SCHEDULE_RANGE || (schedule != HEC_SCHEDULE_GLOBAL && !shaped)))
+        st = build_range(p);
     if (st != HEC_OK) { free_plan(p); return st; }
     *out = p;
     return HEC_OK;
@@ -2593,6 +2599,8 @@ void apply_choice(sptrsv_plan* p, const TuneChoice& c, hec_tune* out) {
         out->blocks_per_sm = c.blocks;
         out->lanes_per_row = c.lpr1;
         out->partitioned = (p->part && c.use_part) ? 1 : 0;
+        out->schedule = out->partitioned ? HEC_SCHEDULE_PART
+                        : p->range && c.use_range ? HEC_SCHEDULE_RANGE : HEC_SCHEDULE_GLOBAL;
     }
 }
 }  // namespace
@@ -2658,8 +2666,8 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
             }
         }
     }
-    if (st == HEC_OK && nrhs == 1 && p->range) {  // the range schedule (its launch shape is its own)
-        const TuneChoice c{bc.threads, bc.blocks, bc.lpr1, 0, 1};
+    if (st == HEC_OK && nrhs == 1 && p->range) {  // the range schedule (launch shape and lanes are its own)
+        const TuneChoice c{bc.threads, bc.blocks, p->range->virt, 0, 1};
         apply_choice(p, c, nullptr);
         float ms = 0.f;
         st = time_it(&ms);

@@ -44,7 +44,9 @@ class HecMatrixInfo(ctypes.Structure):
 
 class HecTune(ctypes.Structure):
     _fields_ = [("block_threads", _i), ("blocks_per_sm", _i), ("wait_cycles", _ll), ("debug_unpublished_row", _i),
-                ("backoff_ns", _i), ("lanes_per_row", _i), ("partitioned", _i)]
+                ("backoff_ns", _i), ("lanes_per_row", _i), ("partitioned", _i), ("schedule", _i)]
+
+SCHEDULES = ("auto", "global", "range", "part")  # HEC_SCHEDULE_*
 
 
 class HecFgmresInfo(ctypes.Structure):
@@ -331,9 +333,13 @@ def hec_to_csr(matrix, levels=None, stream=None):
 
 
 def sptrsv_plan_create(matrix, levels, max_nrhs=1, block_threads=0, blocks_per_sm=0, wait_cycles=0,
-                       debug_unpublished_row=None, backoff_ns=0, lanes_per_row=0):
+                       debug_unpublished_row=None, backoff_ns=0, lanes_per_row=0, schedule="auto", partitioned=False):
+    """Solve plan of one factor.  The range schedule (one launch a sweep) comes with max_nrhs = 1; plans for more
+    right-hand sides sweep single ones with the global schedule.  Takes what sptrsv_autotune returns as
+    keywords and then runs the same schedule (`partitioned` itself is ignored: see sptrsv_plan_partition)."""
     t = HecTune(block_threads, blocks_per_sm, wait_cycles,
-                0 if debug_unpublished_row is None else int(debug_unpublished_row) + 1, backoff_ns, lanes_per_row, 0)
+                0 if debug_unpublished_row is None else int(debug_unpublished_row) + 1, backoff_ns, lanes_per_row, 0,
+                SCHEDULES.index(schedule))
     out = _vp()
     _check(_sptrsv_plan_create(matrix.h, levels.h, int(max_nrhs), ctypes.byref(t), ctypes.byref(out)), "sptrsv_plan_create")
     return Plan(out.value, keep=(matrix, levels))
@@ -368,11 +374,12 @@ _sptrsv_autotune = _sig("sptrsv_autotune", _vp, _i, ctypes.POINTER(HecTune), _vp
 
 
 def sptrsv_autotune(plan, nrhs=1, stream=None):
-    """Times the plan's sweep over candidate launch shapes and keeps the fastest; returns it."""
+    """Times the plan's sweep over candidate launch shapes and schedules and keeps the fastest; returns it.  `schedule`
+    is what now runs: "global", "range" or "part"; the shape is the fastest of the global kernels."""
     t = HecTune()
     _check(_sptrsv_autotune(plan.h, int(nrhs), ctypes.byref(t), _stream(stream)), "sptrsv_autotune")
     return dict(block_threads=t.block_threads, blocks_per_sm=t.blocks_per_sm, lanes_per_row=t.lanes_per_row,
-                partitioned=bool(t.partitioned))
+                partitioned=bool(t.partitioned), schedule=SCHEDULES[t.schedule])
 
 
 def sptrsv_lower(plan, b, x=None, stream=None):
