@@ -255,8 +255,8 @@ int sptrsv_partition_capacity(const sptrsv_plan* p, int threads);
 /* Autotuner: times the plan's own sweep (on a zero right-hand side, nrhs columns) and keeps the
  * fastest of the candidates in the plan; `out` (host, may be NULL) receives the choice.
  * Candidates: launch shapes block_threads in {128, 256} x blocks_per_sm in {2, 4, 8, 16} (those
- * that fit 2048 threads per SM); for nrhs = 1 also lanes per row in {1, 2, 4, 8} (one thread per
- * row against several lanes sharing a long row), the plan's range schedule when it has one
+ * that fit 2048 threads per SM), and 64 x 8 where that is the plan's own; for nrhs = 1 also lanes per row in {1, 2, 4, 8}
+ * (one thread per row against several lanes sharing a long row), the plan's range schedule when it has one
  * (sptrsv_plan_create), and, when the plan has a partition
  * (sptrsv_plan_partition), the partitioned schedule against the best global one (a plan whose
  * global schedule wins keeps its partition unused; partitioning it again re-enables it).

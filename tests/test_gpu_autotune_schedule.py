@@ -45,6 +45,33 @@ def test_report_reproduces_the_choice(case, schedule):
     assert np.max(np.abs(x.cpu().numpy() - ref)) <= 1e-12 * np.max(np.abs(ref))
 
 
+def test_own_shape_is_among_the_candidates():
+    """Eight lanes a row on narrow levels: 64 threads, 8 blocks an SM by default (1838 us an L+U apply; the fastest of the other
+    shapes 1866), which a tuned plan may not lose."""
+    from paper_1606_00541_gb300 import hec
+    A = dev(synth.stencil27_jitter(100, seed=1))
+    T = hec.ilu_factor(*A, k=0)[0].tensors()
+    lv = hec.sptrsv_analyze(T[0], T[1], 0)
+    H = hec.hec_from_csr(*T, levels=lv)
+    b = torch.ones(100 ** 3, dtype=torch.float64, device="cuda")
+    best = {}
+    for name in ("own", "tuned"):
+        plan = hec.sptrsv_plan_create(H, lv, schedule="global")
+        if name == "tuned":
+            hec.sptrsv_autotune(plan, 1)
+        x = hec.sptrsv_lower(plan, b)
+        times = []
+        for _ in range(30):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            hec.sptrsv_lower(plan, b, x)
+            e1.record()
+            e1.synchronize()
+            times.append(e0.elapsed_time(e1))
+        best[name] = min(times)
+    assert best["tuned"] <= 1.01 * best["own"], best
+
+
 def test_unknown_schedule_is_refused():
     from paper_1606_00541_gb300 import hec
     T = dev(oracle.ilu0(synth.poisson2d_5pt(8))[0])
