@@ -298,7 +298,7 @@ def main():
     sched = Schedule(args.sweep, m, devn, torch)
 
     def step(vdt="f32", Lf=L, Uf=U, b=bd, A_=Ad):
-        s = hec.IluSolver(Lf, Uf, A=A_, vdt=vdt)
+        s = hec.IluSolver(Lf, Uf, A=A_, vdt=vdt, **sched.plan_args())
         sched.apply(s, vdt)
         x, info = s.solve(b, restart=RESTART, rtol=RTOL, max_iters=5000)
         return x, info, s
@@ -451,7 +451,7 @@ def precision_times(hec, torch, Ad, L, U, bd, sched):
     out = {}
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     for vdt in ("f64", "f32", "bf16"):
-        s = hec.IluSolver(L, U, A=Ad, vdt=vdt)
+        s = hec.IluSolver(L, U, A=Ad, vdt=vdt, **sched.plan_args())
         sched.apply(s, vdt)
         s.solve(bd, restart=RESTART, rtol=RTOL, max_iters=5000)
         torch.cuda.synchronize()
@@ -474,7 +474,7 @@ def gram_schmidt_times(hec, torch, Ad, L, U, bd, sched):
     try:
         for mode in ("classical", "modified"):
             hec.set_gram_schmidt(mode)
-            s = hec.IluSolver(L, U, A=Ad, vdt="f32")
+            s = hec.IluSolver(L, U, A=Ad, vdt="f32", **sched.plan_args())
             sched.apply(s, "f32")
             s.solve(bd, restart=RESTART, rtol=RTOL, max_iters=5000)
             torch.cuda.synchronize()
@@ -571,8 +571,7 @@ def learned_variant(hec, torch, m, seed=0, crop=32, crops=125, epochs=8, log=Non
     sched = Schedule("part", m, b.device, torch)
     sched.apply(s)
     tuned = s.autotune(1)
-    schedule = ("x-pencil partitioned, %d parts" % sched.nparts if all(t["partitioned"] for t in tuned)
-                else "global") + " (sptrsv_autotune: %s)" % (list(tuned),)
+    schedule = tuned_schedule(tuned, sched.nparts)
     stage = hec.Stage(net, s.A, (m, m, m), torch.as_tensor(lnk, device="cuda"), rho=0.99)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     res = {"train": tinfo, "sweep_schedule": schedule}
@@ -596,9 +595,18 @@ def learned_variant(hec, torch, m, seed=0, crop=32, crops=125, epochs=8, log=Non
 
 
 
+def tuned_schedule(tuned, nparts):
+    """What the autotuned sweeps of a solver run, from its two reports."""
+    names = {"part": "x-pencil partitioned, %d parts" % nparts, "range": "ranges", "global": "global"}
+    kinds = [t["schedule"] for t in tuned]
+    text = names[kinds[0]] if kinds[0] == kinds[1] else "L %s, U %s" % tuple(names[k] for k in kinds)
+    return text + " (sptrsv_autotune: %s)" % (list(tuned),)
+
+
 class Schedule:
     """The single-RHS sweep schedule a solver is given: "global" (the level-ordered kernel over the
-    whole factor) or "part" (x-pencil parts, one resident block each, sptrsv_plan_partition)."""
+    whole factor) or "part" (x-pencil parts, one resident block each, sptrsv_plan_partition).  The
+    default plan's own choice is the range schedule, so "global" is asked for (plan_args)."""
 
     def __init__(self, kind, m, device, torch):
         from paper_1606_00541_gb300 import synth
@@ -606,6 +614,9 @@ class Schedule:
         if kind == "part":
             part, self.nparts = synth.grid_boxes(m, sweep_grid(m))
             self.part = torch.as_tensor(part, device=device)
+
+    def plan_args(self):
+        return {"schedule": "global"} if self.kind == "global" else {}
 
     def apply(self, s, vdt="f32"):
         if self.kind == "part":
@@ -728,6 +739,8 @@ def long_row_variant(hec, torch, hbm, device, m=100, ilut=None):
             key = "one_lane" if lpr == 1 else "autotuned_lanes_%d_%d" % (tuned[0]["lanes_per_row"],
                                                                            tuned[1]["lanes_per_row"])
             res[key] = {"lu_us": ta * 1e6, "lu_gbs": B / ta / 1e9, "frac_hbm": B / ta / 1e9 / hbm}
+            if tuned:
+                res[key]["schedules"] = [t["schedule"] for t in tuned]
             if lpr == 0:
                 s.solve(b, restart=RESTART, rtol=RTOL, max_iters=5000)
                 torch.cuda.synchronize()
