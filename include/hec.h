@@ -194,8 +194,8 @@ typedef struct {
                                an input */
     int schedule;           /* HEC_SCHEDULE_*.  Input: AUTO (0) = the range schedule where it pays and no
                                shape, lanes or backoff is given; GLOBAL = never the range schedule;
-                               RANGE = the range schedule where it pays, also with a shape and lanes
-                               given; PART = as AUTO (the partition itself is given with
+                               RANGE = the range schedule wherever it can run (shared memory, residency,
+                               wait budget), also with a shape and lanes given; PART = as AUTO (the partition itself is given with
                                sptrsv_plan_partition).  Output of sptrsv_autotune: what sweeps of the
                                tuned number of right-hand sides now run.  block_threads and blocks_per_sm then are
                                the fastest shape of the global kernels, which RANGE and PART sweeps do not
@@ -208,10 +208,12 @@ enum { HEC_SCHEDULE_AUTO = 0, HEC_SCHEDULE_GLOBAL = 1, HEC_SCHEDULE_RANGE = 2, H
 /* A solve plan for one triangular factor: its HEC form and level analysis (both borrowed; they
  * must outlive the plan) plus the workspace for up to max_nrhs right-hand sides
  * (1 <= max_nrhs <= 16).  tune may be NULL for defaults.
- * A plan for one right-hand side (max_nrhs = 1) with the default launch shape and lanes per row, or with
- * HEC_SCHEDULE_RANGE, also gets, where it pays and device memory allows, the range schedule: contiguous ranges of original rows, one resident
- * block each with its solution in shared memory, results as the global schedule's bit for bit.  It
- * keeps a copy of the factor's column indices and two n-entry solution buffers. */
+ * A plan for one right-hand side (max_nrhs = 1) with the default launch shape and lanes per row also
+ * gets, where it pays (HEC_SCHEDULE_RANGE: wherever it can run) and device memory allows, the range
+ * schedule: contiguous ranges of original rows, one resident block each with its solution in shared
+ * memory, results as the global schedule's bit for bit.  It keeps a copy of the factor's column indices
+ * and two n-entry solution buffers, also when the plan is partitioned afterwards (HEC_SCHEDULE_GLOBAL
+ * saves a plan that will be partitioned both). */
 hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* lv, int max_nrhs,
                               const hec_tune* tune, sptrsv_plan** out);
 hec_status sptrsv_plan_destroy(sptrsv_plan* p);
@@ -255,9 +257,9 @@ int sptrsv_partition_capacity(const sptrsv_plan* p, int threads);
 /* Autotuner: times the plan's own sweep (on a zero right-hand side, nrhs columns) and keeps the
  * fastest of the candidates in the plan; `out` (host, may be NULL) receives the choice.
  * Candidates: launch shapes block_threads in {128, 256} x blocks_per_sm in {2, 4, 8, 16} (those
- * that fit 2048 threads per SM), and 64 x 8 where that is the plan's own; for nrhs = 1 also lanes per row in {1, 2, 4, 8}
- * (one thread per row against several lanes sharing a long row), the plan's range schedule when it has one
- * (sptrsv_plan_create), and, when the plan has a partition
+ * that fit 2048 threads per SM), and 64 x 8 where that is the plan's own; for nrhs = 1 also lanes per
+ * row in {1, 2, 4, 8} (one thread per row against several lanes sharing a long row), the plan's range
+ * schedule when it has one (sptrsv_plan_create), and, when the plan has a partition
  * (sptrsv_plan_partition), the partitioned schedule against the best global one (a plan whose
  * global schedule wins keeps its partition unused; partitioning it again re-enables it).
  * Results are cached per (rows, slab width, tail entries, levels, value type, nrhs rounded up to

@@ -2311,7 +2311,8 @@ __global__ void k_range_cost(int nlev, int sms, int lanes, const int* __restrict
 //   Long rows: two lanes each, 10 rows of an average level a part (20 rows: 64^3 1569 us).  27-point ILU(0)
 // 16^3 237 / 182 (158 / 109), 33 x 31 x 40 671 / 432 (585 / 329), 64^3 1161 / 1049 (1017 / 744), its ILUT
 // 64^3 1585 / 1129 (1237 / 770); ILU(2) of the 7-point matrix 64^3 1711 / 1328 (1249 / 867).
-hec_status build_range(sptrsv_plan* p) {
+//   forced: without the estimates (HEC_SCHEDULE_RANGE).
+hec_status build_range(sptrsv_plan* p, bool forced) {
     const int kRangeLevelRows = p->lpr1 > 1 ? 10 : 43;
     const hec_matrix* T = p->T;
     const hec_levels* lv = p->lv;
@@ -2390,7 +2391,8 @@ hec_status build_range(sptrsv_plan* p) {
     // kernel only waits for the chunks in flight before its own: its wait must stay well inside the budget
     // (four times the estimated sweep at 2.1 GHz)
     const bool slow = (double)h[4] * 10.0 * 2.1 * 4.0 > (double)p->wait_cycles;
-    if (slow || (long long)h[1] * 10 > entries * 8 || h[4] * (streams ? 150 : 100) > h[5] * 85 ||
+    const bool pays = (long long)h[1] * 10 <= entries * 8 && h[4] * (streams ? 150 : 100) <= h[5] * 85;
+    if (slow || !(pays || forced) ||
         max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
         free_range(R);
         return done(HEC_OK);
@@ -2476,7 +2478,7 @@ HEC_API hec_status sptrsv_plan_create(const hec_matrix* tri, const hec_levels* l
     const bool shaped = tune && (tune->block_threads || tune->blocks_per_sm || tune->backoff_ns || tune->lanes_per_row);
     const int schedule = tune ? tune->schedule : HEC_SCHEDULE_AUTO;
     if (st == HEC_OK && max_nrhs == 1 && (schedule == HEC_SCHEDULE_RANGE || (schedule != HEC_SCHEDULE_GLOBAL && !shaped)))
-        st = build_range(p);
+        st = build_range(p, schedule == HEC_SCHEDULE_RANGE);
     if (st != HEC_OK) { free_plan(p); return st; }
     *out = p;
     return HEC_OK;

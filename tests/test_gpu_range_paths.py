@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from paper_1606_00541_gb300 import synth
+from test_gpu_range import FACTORS, _box
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +35,46 @@ def test_declined_plan_builds_no_tables():
     b = torch.ones(3000, dtype=torch.float64, device="cuda")
     assert launches(hec, lambda: hec.sptrsv_lower(plan, b))[0] == 2  # the global schedule: fill and sweep
     assert own - base == 3
+
+
+PATHS = {  # name: (L and U, slab width)
+    **{name: (lambda hec, make=make, k=k: hec.ilu_factor(*dev(make()), k=k), w) for name, (make, k, w) in FACTORS.items()},
+    "box_w4": (lambda hec: hec.ilu_factor(*dev(_box(19, 23, 17)), k=0), 4),
+    "ilut_w8": (lambda hec: hec.ilut_factor(*dev(_box(19, 23, 17)), p=10, tol=1e-4), 8),  # four partial sums, two slots a wait
+}
+
+
+@pytest.mark.parametrize("vdt", ["f64", "f32"])
+@pytest.mark.parametrize("name", list(PATHS))
+def test_ranges_asked_for_equal_global_bitwise(name, vdt):
+    """Every factor on the range kernels, whether the estimates would choose them or not."""
+    from paper_1606_00541_gb300 import hec
+    make, w = PATHS[name]
+    for uplo, h in enumerate(make(hec)):
+        H, lv = packed(hec, h.tensors(), uplo, w, vdt)
+        solve = (hec.sptrsv_lower, hec.sptrsv_upper)[uplo]
+        n = lv.n
+        plans = [hec.sptrsv_plan_create(H, lv, schedule=s) for s in ("range", "global")]
+        hec.sptrsv_plan_check(plans[0])
+        for seed in range(2):
+            b = torch.as_tensor(synth.uniform_vector(n, seed), device="cuda")
+            (ran, x), (ran2, y) = (launches(hec, lambda: solve(p, b)) for p in plans)
+            assert (ran, ran2) == (1, 2) and torch.equal(x, y)
+        assert hec.hec_sync_status(plans[0]) == hec.OK
+
+
+@pytest.mark.parametrize("case", ["several_ranges", "two_lanes"])
+def test_unpublished_row_ends_the_waits(case):
+    """A row whose word never comes, in a factor of several ranges and in one with two lanes a row: the sweep ends with a
+    timeout, and the next one, of a sound plan, is right."""
+    from paper_1606_00541_gb300 import hec
+    A = synth.poisson2d_5pt(201, 199) if case == "several_ranges" else synth.stencil27_jitter(21, seed=3)
+    T = hec.ilu_factor(*dev(A), k=0)[0].tensors()
+    H, lv = packed(hec, T, 0)
+    n = lv.n
+    b = torch.as_tensor(synth.uniform_vector(n, 3), device="cuda")
+    bad = hec.sptrsv_plan_create(H, lv, schedule="range", wait_cycles=5_000_000, debug_unpublished_row=n // 3)
+    assert launches(hec, lambda: hec.sptrsv_lower(bad, b))[0] == 1
+    assert hec.hec_sync_status(bad) == hec.STATUS_NAMES.index("TIMEOUT")
+    good, ref = (hec.sptrsv_plan_create(H, lv, schedule=s) for s in ("range", "global"))
+    assert torch.equal(hec.sptrsv_lower(good, b), hec.sptrsv_lower(ref, b))
