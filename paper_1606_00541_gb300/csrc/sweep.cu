@@ -1261,21 +1261,6 @@ __global__ void __launch_bounds__(WMAX <= 4 ? 1024 : 512, 1) k_sweep_range(Range
         const int tmax = __reduce_max_sync(kFull, tl);
         slab.wait(xp, p.status, p.budget);
         acc = slab.accumulate(acc, p.w);
-        for (int kb = WMAX; kb < p.w; kb += kTailBatch) {  // wider slabs, kTailBatch slots at a time
-            DepBatchP<XT, AT, kTailBatch> more;
-            more.clear();
-#pragma unroll
-            for (int j = 0; j < kTailBatch; ++j) {
-                const int k = kb + j;
-                if (act && k < p.w) {
-                    const long s = (long)k * p.ld + r;
-                    range_set(more, j, sbase, __ldg(p.ell_col + s), ldv<VT, AT>(ev + s));
-                }
-            }
-            more.poll(xp);
-            more.wait(xp, p.status, p.budget);
-            acc = more.accumulate(acc);
-        }
         for (int tb = 0; tb < tmax; tb += kTailBatch) {
             DepBatchP<XT, AT, kTailBatch> tail;
             tail.clear();
@@ -1690,7 +1675,7 @@ template <typename VT, typename XT>
 const void* range_kernel(int w, int v) {
     if (v == 2) return (const void*)k_sweep_range_lpr<VT, XT, 2, 4>;
     if (v == 4) return w <= 8 ? (const void*)k_sweep_range_lpr<VT, XT, 4, 4> : (const void*)k_sweep_range_lpr<VT, XT, 4, 8>;
-    if (v == 8) return w <= 8 ? (const void*)k_sweep_range_lpr<VT, XT, 8, 4> : (const void*)k_sweep_range_lpr<VT, XT, 8, 8>;
+    if (v == 8) return (const void*)k_sweep_range_lpr<VT, XT, 8, 8>;
     return w <= 3   ? (const void*)k_sweep_range<VT, XT, 3>
            : w <= 4 ? (const void*)k_sweep_range<VT, XT, 4>
                     : (const void*)k_sweep_range<VT, XT, 8>;

@@ -89,11 +89,6 @@ __device__ __forceinline__ float wait_f32(const float* p, int* status, long long
     if (v == kSent32) v = spin_until_not<unsigned int>(p, kSent32, status, budget, LoadU32());
     return __uint_as_float(v);
 }
-__device__ __forceinline__ int wait_i32(const int* p, int* status, long long budget) {
-    unsigned int v = ld_relaxed_u32(p);
-    if (v == (unsigned)kSentI) v = spin_until_not<unsigned int>(p, (unsigned)kSentI, status, budget, LoadU32());
-    return (int)v;
-}
 
 __device__ __forceinline__ void publish_f64(double* p, double x) {
     unsigned long long u = (unsigned long long)__double_as_longlong(x);
