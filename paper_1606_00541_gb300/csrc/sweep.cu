@@ -2653,13 +2653,14 @@ HEC_API hec_status sptrsv_autotune(sptrsv_plan* p, int nrhs, hec_tune* out, void
             }
         }
     }
-    // the plan's own shape where it is none of these (see sweep_shape)
+    // the plan's own shape where it is none of these (see sweep_shape); another has to be faster by more than three
+    // sweeps' times differ by themselves
     if (st == HEC_OK && nrhs == 1 && !was_shaped && saved.lpr1 >= 4) {
         const TuneChoice c{64, 8, saved.lpr1, 0, 0};
         apply_choice(p, c, nullptr);
         float ms = 0.f;
         st = time_it(&ms);
-        if (st == HEC_OK && ms < best) { best = ms; bc = c; }
+        if (st == HEC_OK && ms < 1.02f * best) { best = ms; bc = c; }
     }
     if (st == HEC_OK && nrhs == 1 && p->range) {  // the range schedule (launch shape and lanes are its own)
         const TuneChoice c{bc.threads, bc.blocks, p->range->virt, 0, 1};
