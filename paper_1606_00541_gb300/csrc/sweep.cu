@@ -2146,13 +2146,16 @@ hec_status build_partition(sptrsv_plan* p, const int* part, int nparts, cudaStre
 namespace {
 // what the choice needs to know of the columns: counts[0] += entries whose row is in another range, counts[1] +=
 // the longest tail (without the diagonal) of each 32 rows, in waits of `batch` entries, counts[2] += how many 32
-// rows have a tail
-__global__ void k_range_count(int n, int ld, int w, int rows, int batch, const int* __restrict__ ec,
+// rows have a tail.  Of every `step`-th 256 rows of the level order: the choice needs shares, not totals, and 256 K
+// rows give them
+constexpr int kRangeSample = 1024;
+__global__ void k_range_count(int n, int ld, int w, int rows, int batch, int step, const int* __restrict__ ec,
                               const int* __restrict__ tp, const int* __restrict__ tc, const int* __restrict__ iperm,
                               unsigned long long* counts) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const long at = (long)blockIdx.x * step * blockDim.x + threadIdx.x;
     int cross = 0, waits = 0;
-    if (r < n) {
+    if (at < n) {
+        const int r = (int)at;
         const int q = __ldg(iperm + r) / rows, t0 = __ldg(tp + r), t1 = __ldg(tp + r + 1) - 1;
         waits = (t1 - t0 + batch - 1) / batch;
         for (int k = 0; k < w; ++k) {
@@ -2348,8 +2351,9 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     k_range_chunk_counts<<<g, 128, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr, most, total,
                                            counts);
     k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, R->lanes, lv->level_ptr, most, counts + 4);
-    k_range_count<<<(n + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, R->lanes == 1 ? kTailBatch : virt, T->ell_col, T->tptr,
-                                                  T->tcol, lv->iperm, counts + 1);
+    const int blocks = (n + 255) / 256, step = (blocks + kRangeSample - 1) / kRangeSample;
+    k_range_count<<<(blocks + step - 1) / step, 256, 0, s>>>(n, T->ld, T->w, R->rows, R->lanes == 1 ? kTailBatch : virt, step,
+                                                             T->ell_col, T->tptr, T->tcol, lv->iperm, counts + 1);
     count_launch(3);
     unsigned long long h[kCounts] = {};
     if (cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -2376,7 +2380,7 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     // kernel only waits for the chunks in flight before its own: its wait must stay well inside the budget
     // (four times the estimated sweep at 2.1 GHz)
     const bool slow = (double)h[4] * 10.0 * 2.1 * 4.0 > (double)p->wait_cycles;
-    const bool pays = (long long)h[1] * 10 <= entries * 8 && h[4] * (streams ? 150 : 100) <= h[5] * 85;
+    const bool pays = (long long)h[1] * step * 10 <= entries * 8 && h[4] * (streams ? 150 : 100) <= h[5] * 85;
     if (slow || !(pays || forced) ||
         max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
         free_range(R);
