@@ -136,7 +136,7 @@ __global__ void k_check_part_chunks(int nparts, const int* __restrict__ part_row
 }
 
 // the range schedule: every row in exactly one chunk (`seen`), of its range and of one level, a range's
-// chunks in level order; the columns those of the factor in original numbering
+// chunks in level order; the coded columns those of the factor
 __global__ void k_check_range_chunks(int n, int nparts, int rows, const int* __restrict__ part_chunk,
                                      const int2* __restrict__ ch, int cap, int rpw, const int* __restrict__ iperm,
                                      const int* __restrict__ lp, int nlev, unsigned* seen, unsigned* res) {

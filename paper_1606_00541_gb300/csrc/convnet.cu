@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(tc_threads(EXP), 2)
 // dZ = dA masked by the layer's ReLU (mask = its output) when mask is given.
 //   A block takes the tiles blockIdx.x, + gridDim.x, ... (32 x 4 x 1 voxels with a 34 x 6 x 3 halo)
 // and keeps its sums in registers, so 27.7 KB of partial sums are written once per block
-// (kWgradBlocks an SM) instead of once per tile: at 8 x 32^3 voxels 17 MB a layer instead of 57 MB,
+// (kWgradBlocks an SM) instead of once per tile: at 8 x 32^3 voxels 12.6 MB a layer instead of 57 MB,
 // and as much less for the reduction to read.  Warp w owns the taps w, w + 4, ...; a tile's products
 // are summed by the tensor cores from zero and added to the running sums in FP32.  Both operands are
 // voxel-major in shared memory and are transposed by ldmatrix; the dZ fragments of a tile (8 steps of

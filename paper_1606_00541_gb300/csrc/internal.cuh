@@ -125,7 +125,8 @@ struct hec_part_data {
 // The default schedule of single-right-hand-side sweeps (see sweep.cu, "ranges"): part q owns the
 // original rows [q * rows, (q + 1) * rows).  Inside a level the level order ascends (descends, for an
 // upper factor) in the original row, so a part's rows of a level are consecutive rows of the factor as
-// it is packed, and only a chunk table and the columns in original numbering are added.
+// it is packed, and only a chunk table and a coded copy of the columns are added (a word of the range's own
+// solution, or the level-ordered row of another range).
 struct hec_range_data {
     int nparts = 0, rows = 0, threads = 0, cap_chunks = 0;
     int lanes = 1;              // lanes per row: chunks hold up to 32 / lanes rows

@@ -99,9 +99,10 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // The warp waits, converged, until every lane's pending dependency words have been published.  A poll
 // issues the loads of all outstanding words before it looks at the first (ld_relaxed_if): one L2 round
-// trip a poll instead of one a word.  Default plans, word by word / this: L+U apply of the 7-point 100^3
-// ILU(0), FP64 704 / 546 us; 64 x 64 grid, 234 / 162 us; 16 right-hand sides on 64 Schwarz boxes of 128^3,
-// FP32 648 / 590 us.
+// trip a poll instead of one a word, and as many more loads in flight, which bounds how many warps may
+// wait at once (sweep_shape).  Global kernels with all the warps that fit, word by word / this: L+U apply of the
+// 7-point 100^3 ILU(0), FP64 704 / 546 us; 64 x 64 grid, 234 / 162 us; 16 right-hand sides on 64 Schwarz
+// boxes of 128^3, FP32 648 / 590 us.
 // pending: bit k set = slot k of this lane still outstanding.  Polls are issued for all
 // outstanding slots at once.  Returns false (and records DEV_TIMEOUT) when the budget runs out.
 template <typename XT, int NS>
@@ -292,6 +293,8 @@ __global__ void __launch_bounds__(256) k_sweep(SweepParams p) {
 // The partial sums are combined by an xor butterfly, which gives every lane of the group the
 // same bits; the fixed pairing makes the result deterministic (it differs from the one-lane
 // kernel only in summation order).
+// BF16 rows of two lanes keep six blocks an SM (40 registers): wide levels are bound by bandwidth (eight colours
+// of the 27-point 100^3, 44 registers and five blocks / this: 158 / 141 us).
 template <typename VT, typename XT, int LPR, int SPL, int TB>
 __global__ void __launch_bounds__(256, LPR == 2 && sizeof(VT) == 2 ? 6 : 0) k_sweep_lpr(SweepParams p) {
     typedef typename Acc<XT>::T AT;
@@ -2289,16 +2292,16 @@ __global__ void k_range_cost(int nlev, int sms, int lanes, const int* __restrict
 //   Parts: kRangeLevelRows rows of an average level each.  More parts cross more boundaries on the
 // dependency chain, fewer make a level's chunks queue in a block (24 / 43 / 64 rows: 50^3 151 / 129 / 151 us,
 // 100^3 457 / 359 / 341, 128^3 512 / 487 / 484).
-// L+U apply of ILU(0), global / range schedule, FP64 (FP32): 5-point 64 x 64 166 / 79 us (132 / 60),
-// 150 x 150 374 / 185 (313 / 128), 1000 x 1000 2810 / 1190 (2250 / 885); 7-point 16^3 80 / 42 (58 / 30),
-// 31 x 37 x 29 161 / 80 (130 / 62), 50^3 245 / 129 (191 / 102), 64^3 323 / 172 (244 / 136), 100^3 548 / 359
-// (423 / 290), 128^3 723 / 486 (542 / 413), 160^3 937 / 726 (684 / 580); 576 Schwarz boxes of 128^3
+// L+U apply of ILU(0), global / range schedule, FP64 (FP32): 5-point 64 x 64 169 / 86 us (140 / 60),
+// 150 x 150 390 / 195 (337 / 135), 1000 x 1000 2613 / 1131 (2122 / 896); 7-point 16^3 95 / 57 (75 / 46),
+// 31 x 37 x 29 178 / 95 (136 / 75), 50^3 257 / 145 (203 / 115), 64^3 326 / 186 (252 / 148), 100^3 548 / 367
+// (425 / 295), 128^3 723 / 490 (548 / 407), 160^3 951 / 725 (716 / 571); 576 Schwarz boxes of 128^3
 // 201 / 162 (177 / 116).  Where the estimate keeps the global one: 64 boxes 239 / 357 (193 / 270), FP32
 // 200^3 (921 / 926), random rows of six entries 248 / 390.  More than four slots, global / range: ILU(1)
-// of the 7-point matrix 40^3 431 / 297 (307 / 210), 64^3 726 / 467 (588 / 331), 100^3 1178 / 1009.
+// of the 7-point matrix 40^3 440 / 308 (326 / 214), 64^3 717 / 473 (523 / 330), 100^3 1164 / 1020 (858 / 745).
 //   Long rows: two lanes each, 10 rows of an average level a part (20 rows: 64^3 1569 us).  27-point ILU(0)
-// 16^3 237 / 182 (158 / 109), 33 x 31 x 40 671 / 432 (585 / 329), 64^3 1161 / 1049 (1017 / 744), its ILUT
-// 64^3 1585 / 1129 (1237 / 770); ILU(2) of the 7-point matrix 64^3 1711 / 1328 (1249 / 867).
+// 16^3 246 / 198 (165 / 124), 33 x 31 x 40 646 / 450 (478 / 344), 64^3 1095 / 1070 (933 / 714), its ILUT
+// 64^3 1381 / 1030 (996 / 743); ILU(2) of the 7-point matrix 64^3 1647 / 1318 (1138 / 911).
 //   forced: without the estimates (HEC_SCHEDULE_RANGE).
 hec_status build_range(sptrsv_plan* p, bool forced) {
     const int kRangeLevelRows = p->lpr1 > 1 ? 10 : 43;
