@@ -14,9 +14,10 @@
 // W consecutive rows are in flight, half a plane of a 100^3 grid, whose wavefront keeps a few dozen of
 // the 4,864 warps busy.  Groups put a dozen planes in flight, and a run held by a group holds back no row
 // (each waits for the row before it anyway), while its warps work on the earlier pivots of the rows
-// ahead.  With enough rows at work the FP64 unit is the bound (16 SM-cycles a warp instruction): per row
-// about 25 divisions and 40 ranked candidates, so the ranking compares magnitudes as integers and the
-// division takes five FP64 instructions (div_by).  27-point 100^3 / 7-point 100^3: 45.2 / 37.7 ms with
+// ahead.  With enough rows at work the FP64 unit counts (16 SM-cycles a warp instruction): per row
+// about 25 divisions and 40 ranked candidates (268 FP64 warp instructions are left: the unit is busy 43 % of the time
+// on 64^3 and, by that count, 62 % on 100^3; the rest is a pivot's flag and the loads behind it, one pivot after the other),
+// so the ranking compares magnitudes as integers and the division takes five FP64 instructions (div_by).  27-point 100^3 / 7-point 100^3: 45.2 / 37.7 ms with
 // FP64 compares and __ddiv_rn, 28.5 / 26.6 with integer compares, 22.0 / 23.2 with both.
 //   The groups, before that.  ILUT(10, 1e-3) of the 27-point stencil on 100^3 / 64^3 and of the 7-point matrix on 100^3:
 // row by row 167.6 / 45.1 / 189.0 ms, groups of 8 warps 45.2 / 17.2 / 37.7 (1 warp 100 / 39.7 / 110,
