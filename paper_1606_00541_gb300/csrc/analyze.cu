@@ -222,11 +222,14 @@ __global__ void k_digit_scatter(int n, SortIn in, int shift, int bits, int ntile
     const unsigned lt = (1u << lane) - 1u;
     const long t0 = (long)tile * kTileItems;
     long t = t0 + lane;
-    int kn = t < n ? in.k(n, t) : 0;  // one step ahead: its load overlaps the ranking
+    int kn = t < n ? in.k(n, t) : 0, vn = t < n ? in.v(n, t) : 0;  // one step ahead: the loads overlap the ranking
     for (int r = 0; r < kTileItems && t0 + r < n; r += 32, t += 32) {
         const bool ok = t < n;
-        const int k = kn;
-        if (t + 32 < n) kn = in.k(n, t + 32);
+        const int k = kn, v = vn;
+        if (t + 32 < n) {
+            kn = in.k(n, t + 32);
+            vn = in.v(n, t + 32);
+        }
         const int d = ok ? ((k >> shift) & (digits - 1)) : digits + lane;  // invalid lanes get unique digits
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const int rank = __popc(peers & lt);
@@ -235,7 +238,6 @@ __global__ void k_digit_scatter(int n, SortIn in, int shift, int bits, int ntile
         if (ok && rank == 0) base[d] += __popc(peers);
         __syncwarp();
         if (ok) {
-            const int v = in.v(n, t);
             if (okey) okey[pos] = k;
             oval[pos] = v;
             if (inv) inv[v] = pos;
