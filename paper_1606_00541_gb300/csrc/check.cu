@@ -163,14 +163,14 @@ __global__ void k_check_range_chunks(int n, int nparts, int rows, const int* __r
         }
     }
 }
-__global__ void k_check_range_cols(int n, int w, int ld, int rows, const unsigned* __restrict__ seen,
+__global__ void k_check_range_cols(int n, int w, int ld, int rows, int pad, const unsigned* __restrict__ seen,
                                    const int* __restrict__ ec, const int* __restrict__ tp, const int* __restrict__ tc,
                                    const int* __restrict__ oc, const int* __restrict__ otc, const int* __restrict__ iperm,
                                    unsigned* res) {
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
         if (!((seen[r >> 5] >> (r & 31)) & 1u)) fail(res, 8, r);
         const int q = iperm[r] / rows;
-        auto code = [&](int c) { return iperm[c] / rows == q ? -2 - (iperm[c] - q * rows) : c; };
+        auto code = [&](int c) { return iperm[c] / rows == q ? -2 - range_slot(iperm[c] - q * rows, pad) : c; };
         for (int k = 0; k < w; ++k) {
             const int c = ec[(long)k * ld + r];
             if (oc[(long)k * ld + r] != (c < 0 ? -1 : code(c))) fail(res, 8, r);
@@ -238,7 +238,7 @@ HEC_API hec_status sptrsv_plan_check(const sptrsv_plan* p, void* stream) {
             cudaMemsetAsync(seen, 0, sizeof(unsigned) * ((size_t)(n + 31) / 32), s);
             k_check_range_chunks<<<R->nparts, 128, 0, s>>>(n, R->nparts, R->rows, R->part_chunk, R->chunks, R->cap_chunks, 32 / R->lanes,
                                                            lv->iperm, lv->level_ptr, lv->nlev, seen, res);
-            k_check_range_cols<<<g, 256, 0, s>>>(n, T->w, T->ld, R->rows, seen, T->ell_col, T->tptr, T->tcol, R->ell_col, R->tcol,
+            k_check_range_cols<<<g, 256, 0, s>>>(n, T->w, T->ld, R->rows, R->pad, seen, T->ell_col, T->tptr, T->tcol, R->ell_col, R->tcol,
                                                  lv->iperm, res);
             count_launch(2);
         }

@@ -122,6 +122,9 @@ struct hec_part_data {
     int* bidx_perm = nullptr;   // [n] plan row -> row of b for sptrsv_lower / sptrsv_upper (iperm[rowg])
 };
 
+// the place of word s (an original row less the range's first) in the range's shared solution
+__host__ __device__ inline int range_slot(int s, int pad) { return s + (((s >> 5) + (s >> 10)) & -pad); }
+
 // The default schedule of single-right-hand-side sweeps (see sweep.cu, "ranges"): part q owns the
 // original rows [q * rows, (q + 1) * rows).  Inside a level the level order ascends (descends, for an
 // upper factor) in the original row, so a part's rows of a level are consecutive rows of the factor as
@@ -130,8 +133,9 @@ struct hec_part_data {
 struct hec_range_data {
     int nparts = 0, rows = 0, threads = 0, cap_chunks = 0;
     int lanes = 1;              // lanes per row: chunks hold up to 32 / lanes rows
+    int pad = 0;                // 1: a word left out after every 32, and after every 1024, of the shared solution
     int virt = 1;               // lanes per row of the global kernel whose sums it reproduces
-    int* ell_col = nullptr;     // [w * ld] the slab's columns: -1 empty, -2 - s word s of the range, else the row
+    int* ell_col = nullptr;     // [w * ld] the slab's columns: -1 empty, -2 - s place s of the range, else the row
     int* tcol = nullptr;        // [tail_nnz] the tail's
     int2* chunks = nullptr;     // (first level-ordered row, rows), part by part in level order
     int* part_chunk = nullptr;  // [nparts + 1]

@@ -1122,7 +1122,7 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_part(PartParams p) {
 // shared memory at (original row - q * rows).  Inside a level the level order follows the original row,
 // so a range's rows of a level are consecutive rows of the packed factor: the kernel reads the slab as
 // it is, and needs only its own chunk table and the columns coded by where their words are: -2 - s for
-// word s of the range's shared solution, the level-ordered row for a row of another range, whose word
+// place s (range_slot) of the range's shared solution, the level-ordered row for a row of another range, whose word
 // is polled in global memory (level order keeps a chunk's words in a few sectors).
 // Every row adds its entries in the order of k_sweep, so results are the same bit for bit.
 //   What bounds it is the latency of a level, as in the other sweeps: 0.3 to 0.6 us where k_sweep takes
@@ -1131,7 +1131,7 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_part(PartParams p) {
 //   Both word buffers and the flag that says which one this sweep polls live on the device: the block
 // that finishes last turns the flag, so no fill launch is needed and a captured graph can be replayed.
 struct RangeParams {
-    int n, ld, w, rows;
+    int n, ld, w, rows, pad;
     const int* __restrict__ ell_col;  // coded (see above)
     const void* __restrict__ ell_val;
     const int* __restrict__ tptr;
@@ -1155,15 +1155,16 @@ struct RangeParams {
     int b32, x32;
 };
 
-// of one lane's row: its original number, the row of b it reads, the row of x it writes (-1: none)
+// of one lane's row: its place in the shared solution, the row of b it reads, the row of x it writes (-1: none)
 struct RangeIdx {
-    int id, gr, sr;
-    __device__ __forceinline__ void load(const RangeParams& p, int2 ch, int rsub) {
-        id = sr = -1;
-        gr = 0;
+    int slot, gr, sr;
+    __device__ __forceinline__ void load(const RangeParams& p, int2 ch, int rsub, int lo) {
+        sr = -1;
+        slot = gr = 0;
         if (rsub < ch.y) {
             const int r = ch.x + rsub;
-            id = __ldg(p.iperm + r);
+            const int id = __ldg(p.iperm + r);
+            slot = range_slot(id - lo, p.pad);
             gr = p.gather == p.iperm ? id : p.gather ? __ldg(p.gather + r) : r;
             sr = p.scatter == p.iperm ? id : p.scatter ? __ldg(p.scatter + r) : r;
         }
@@ -1227,7 +1228,7 @@ __global__ void __launch_bounds__(WMAX <= 4 ? 1024 : 512, 1) k_sweep_range(Range
     const unsigned int sbase = (unsigned int)__cvta_generic_to_shared(smem_raw);
     const int lo = blockIdx.x * p.rows, hi = min(p.n, lo + p.rows);
     const int turn = __ldcg(p.state);  // turned by the last block to finish, when every block has read it
-    for (int i = threadIdx.x; i < hi - lo; i += blockDim.x) sxp[i] = W::kSent;
+    for (int i = threadIdx.x; i < range_slot(hi - lo, p.pad); i += blockDim.x) sxp[i] = W::kSent;
     __syncthreads();
     const int c0 = __ldg(p.part_chunk + blockIdx.x), c1 = __ldg(p.part_chunk + blockIdx.x + 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -1238,8 +1239,8 @@ __global__ void __launch_bounds__(WMAX <= 4 ? 1024 : 512, 1) k_sweep_range(Range
     int c = c0 + warp;
     int2 ch = chunk(c), ch1 = chunk(c + nwarps), ch2 = chunk(c + 2 * nwarps);
     RangeIdx ix, ix1;
-    ix.load(p, ch, lane);
-    ix1.load(p, ch1, lane);
+    ix.load(p, ch, lane, lo);
+    ix1.load(p, ch1, lane, lo);
     RangeRow<VT, XT, AT, WMAX> row, nxt;
     if (PF) nxt.load(p, ch, lane, ix.gr);
     for (; c < c1; c += nwarps) {
@@ -1250,7 +1251,7 @@ __global__ void __launch_bounds__(WMAX <= 4 ? 1024 : 512, 1) k_sweep_range(Range
         } else {
             row.load(p, ch, lane, ix.gr);
         }
-        ix2.load(p, ch2, lane);
+        ix2.load(p, ch2, lane, lo);
         const int2 ch3 = chunk(c + 3 * nwarps);
         const int r = ch.x + lane;
         const bool act = lane < ch.y;
@@ -1279,7 +1280,7 @@ __global__ void __launch_bounds__(WMAX <= 4 ? 1024 : 512, 1) k_sweep_range(Range
         if (act && r != p.skip_row) {
             WT wv = sizeof(XT) == 8 ? (WT)__double_as_longlong((double)(XT)xr) : (WT)__float_as_uint((float)(XT)xr);
             if (wv == W::kSent) wv = sizeof(XT) == 8 ? (WT)0x7FF8000000000000ull : (WT)0x7FC00000u;
-            *(volatile WT*)(sxp + (ix.id - lo)) = wv;  // consumers in this range
+            *(volatile WT*)(sxp + ix.slot) = wv;  // consumers in this range
             publish_x(xp + r, (XT)xr);                 // consumers in other ranges
         }
         if (act && ix.sr >= 0) st_sol(p.x, p.x32, (long)ix.sr * p.ldx, xr);
@@ -1315,7 +1316,7 @@ __global__ void __launch_bounds__(512, 1) k_sweep_range_lpr(RangeParams p) {
     const unsigned int sbase = (unsigned int)__cvta_generic_to_shared(smem_raw);
     const int lo = blockIdx.x * p.rows, hi = min(p.n, lo + p.rows);
     const int turn = __ldcg(p.state);
-    for (int i = threadIdx.x; i < hi - lo; i += blockDim.x) sxp[i] = W::kSent;
+    for (int i = threadIdx.x; i < range_slot(hi - lo, p.pad); i += blockDim.x) sxp[i] = W::kSent;
     __syncthreads();
     const int c0 = __ldg(p.part_chunk + blockIdx.x), c1 = __ldg(p.part_chunk + blockIdx.x + 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -1327,7 +1328,7 @@ __global__ void __launch_bounds__(512, 1) k_sweep_range_lpr(RangeParams p) {
     int c = c0 + warp;
     int2 ch = chunk(c), ch1 = chunk(c + nwarps);
     RangeIdx ix;
-    ix.load(p, ch, rsub);
+    ix.load(p, ch, rsub, lo);
     for (; c < c1; c += nwarps) {
         const int2 ch2 = chunk(c + 2 * nwarps);
         RangeIdx ix1;
@@ -1356,7 +1357,7 @@ __global__ void __launch_bounds__(512, 1) k_sweep_range_lpr(RangeParams p) {
                     range_set(slab, j, sbase, __ldg(p.ell_col + s), ldv<VT, AT>(ev + s));
                 }
             }
-            if (ib == 0) ix1.load(p, ch1, rsub);
+            if (ib == 0) ix1.load(p, ch1, rsub, lo);
             slab.wait(xp, p.status, p.budget);
 #pragma unroll
             for (int j = 0; j < NS; ++j) {
@@ -1364,7 +1365,7 @@ __global__ void __launch_bounds__(512, 1) k_sweep_range_lpr(RangeParams p) {
                 acc[j % NA] = fma(-slab.v[j], (AT)W::val(slab.raw[j]), acc[j % NA]);
             }
         }
-        if (p.w == 0) ix1.load(p, ch1, rsub);
+        if (p.w == 0) ix1.load(p, ch1, rsub, lo);
         const int tmax = __reduce_max_sync(kFull, tl);
         for (int tb = 0; tb < tmax; tb += V) {  // V tail entries of a row at a time
             DepBatchP<XT, AT, NA> tail;
@@ -1389,7 +1390,7 @@ __global__ void __launch_bounds__(512, 1) k_sweep_range_lpr(RangeParams p) {
             if (r != p.skip_row) {
                 WT wv = sizeof(XT) == 8 ? (WT)__double_as_longlong((double)(XT)xr) : (WT)__float_as_uint((float)(XT)xr);
                 if (wv == W::kSent) wv = sizeof(XT) == 8 ? (WT)0x7FF8000000000000ull : (WT)0x7FC00000u;
-                *(volatile WT*)(sxp + (ix.id - lo)) = wv;
+                *(volatile WT*)(sxp + ix.slot) = wv;
                 publish_x(xp + r, (XT)xr);
             }
             if (ix.sr >= 0) st_sol(p.x, p.x32, (long)ix.sr * p.ldx, xr);
@@ -1741,6 +1742,7 @@ hec_status sweep(const sptrsv_plan* pl, int nrhs, const double* b, int ldb, cons
         rp.ld = T->ld;
         rp.w = T->w;
         rp.rows = R->rows;
+        rp.pad = R->pad;
         rp.ell_col = R->ell_col;
         rp.ell_val = T->ell_val;
         rp.tptr = T->tptr;
@@ -1768,7 +1770,7 @@ hec_status sweep(const sptrsv_plan* pl, int nrhs, const double* b, int ldb, cons
         void* tok = nullptr;
         profile_begin(s, &tok);
         HEC_CUDA(cudaLaunchCooperativeKernel(range_kernel(T, R->virt), dim3(R->nparts), dim3(R->threads), args,
-                                             (size_t)R->rows * work_size(T->vdt), s));
+                                             (size_t)range_slot(R->rows, R->pad) * work_size(T->vdt), s));
         profile_end(s, tok);
         count_launch();
         return HEC_OK;
@@ -2149,16 +2151,22 @@ hec_status build_partition(sptrsv_plan* p, const int* part, int nparts, cudaStre
 namespace {
 // what the choice needs to know of the columns: counts[0] += entries whose row is in another range, counts[1] +=
 // the longest tail (without the diagonal) of each 32 rows, in waits of `batch` entries, counts[2] += how many 32
-// rows have a tail.  Of every `step`-th 256 rows of the level order: the choice needs shares, not totals, and 256 K
-// rows give them
+// rows have a tail, counts[5] and counts[6] += for each row, the rows of its chunk whose word is in the same bank of
+// the shared solution, without and with padding (banks: of 8-byte words 16, of 4-byte words 32).  Of every `step`-th
+// 256 rows of the level order: the choices need shares, not totals, and 256 K rows give them
 constexpr int kRangeSample = 1024;
-__global__ void k_range_count(int n, int ld, int w, int rows, int batch, int step, const int* __restrict__ ec,
+__global__ void k_range_count(int n, int ld, int w, int rows, int batch, int step, int banks, const int* __restrict__ ec,
                               const int* __restrict__ tp, const int* __restrict__ tc, const int* __restrict__ iperm,
-                              unsigned long long* counts) {
+                              const int* __restrict__ level, unsigned long long* counts) {
     const long at = (long)blockIdx.x * step * blockDim.x + threadIdx.x;
     int cross = 0, waits = 0;
+    unsigned long long chunk = ~0ull;  // range and level
+    int word = threadIdx.x & 31;
     if (at < n) {
         const int r = (int)at;
+        const int i = __ldg(iperm + r);
+        word = i % rows;
+        chunk = ((unsigned long long)__ldg(level + i) << 32) | (unsigned)(i / rows);
         const int q = __ldg(iperm + r) / rows, t0 = __ldg(tp + r), t1 = __ldg(tp + r + 1) - 1;
         waits = (t1 - t0 + batch - 1) / batch;
         for (int k = 0; k < w; ++k) {
@@ -2169,7 +2177,13 @@ __global__ void k_range_count(int n, int ld, int w, int rows, int batch, int ste
     }
     cross = __reduce_add_sync(0xffffffffu, cross);
     waits = __reduce_max_sync(0xffffffffu, waits);
+    const unsigned same = __match_any_sync(0xffffffffu, chunk);
+    const int c0 = __popc(same & __match_any_sync(0xffffffffu, word % banks));
+    const int c1 = __popc(same & __match_any_sync(0xffffffffu, range_slot(word, 1) % banks));
+    const int plain = __reduce_add_sync(0xffffffffu, c0), padded = __reduce_add_sync(0xffffffffu, c1);
     if ((threadIdx.x & 31) == 0) {
+        atomicAdd(counts + 5, (unsigned long long)plain);
+        atomicAdd(counts + 6, (unsigned long long)padded);
         if (cross) atomicAdd(counts, (unsigned long long)cross);
         if (waits) {
             atomicAdd(counts + 1, (unsigned long long)waits);
@@ -2178,14 +2192,14 @@ __global__ void k_range_count(int n, int ld, int w, int rows, int batch, int ste
     }
 }
 // the columns of slab and tail coded by where their words are (see RangeParams)
-__global__ void k_range_cols(int n, int ld, int w, int rows, const int* __restrict__ ec, const int* __restrict__ tp,
+__global__ void k_range_cols(int n, int ld, int w, int rows, int pad, const int* __restrict__ ec, const int* __restrict__ tp,
                              const int* __restrict__ tc, const int* __restrict__ iperm, int* oec, int* otc) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r < n) {
         const int q = __ldg(iperm + r) / rows;
         auto code = [&](int c) {
             const int j = __ldg(iperm + c);
-            return j / rows == q ? -2 - (j - q * rows) : c;
+            return j / rows == q ? -2 - range_slot(j - q * rows, pad) : c;
         };
         for (int k = 0; k < w; ++k) {
             const long s = (long)k * ld + r;
@@ -2229,7 +2243,7 @@ __global__ void k_range_chunk_counts(int n, int nlev, int nparts, int rows, int 
     atomicAdd(total + q, cnt);
 }
 // the chunk table, a block per part: the parts before it by their totals, its levels by a scan
-constexpr int kRangeTableThreads = 256;
+constexpr int kRangeTableThreads = 1024;  // thousands of levels, few parts (a 2D grid): its searches are the time
 __global__ void __launch_bounds__(kRangeTableThreads) k_range_chunks(int n, int nlev, int nparts, int rows, int rpw, int uplo,
                                                                      const int* __restrict__ iperm,
                                                                      const int* __restrict__ level_ptr,
@@ -2312,7 +2326,10 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     if (n == 0 || sms == 0 || T->w > (virt > 1 ? 3 * virt : 8)) return HEC_OK;  // the slots the kernels take
     const size_t ws = work_size(T->vdt);
     const long avg = (n + nlev - 1) / nlev;
-    long need = (long)((ws * (size_t)n + kRangeSmem - 1) / kRangeSmem);
+    // ranges of a size that leaves room for padding (below), where an SM each has it
+    const long words = (long)(kRangeSmem / ws), rooms = words * 1024 / 1057;
+    long need = (n + rooms - 1) / rooms;
+    if (need > sms) need = (n + words - 1) / words;
     long parts = std::max(need, std::min((avg + kRangeLevelRows / 2) / kRangeLevelRows, (long)sms));
     parts = std::max(1L, std::min(parts, (long)n));
     if (parts > sms || parts * nlev > 4L * n + 1024) return HEC_OK;
@@ -2331,7 +2348,7 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     }
     // The choice comes before any table of the size of the factor: counts of the chunks and a pass over the columns, in one
     // block of memory.  counts: nonempty (part, level) pairs; entries in another range; waits for tails by 32 rows, and such
-    // 32 rows; costs
+    // 32 rows; costs; rows in the same bank without and with padding
     unsigned long long* counts = nullptr;
     cudaStream_t s = 0;
     auto done = [&](hec_status e) {
@@ -2343,7 +2360,7 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
         }
         return e;
     };
-    constexpr int kCounts = 6;
+    constexpr int kCounts = 8;
     const size_t scratch = kCounts * sizeof(*counts) + sizeof(int) * ((size_t)nlev + R->nparts);
     hec_status st = dmalloc((void**)&counts, scratch);
     if (st) return done(st);
@@ -2356,7 +2373,8 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     k_range_cost<<<std::min(64, nlev / 256 + 1), 256, 0, s>>>(nlev, sms, R->lanes, lv->level_ptr, most, counts + 4);
     const int blocks = (n + 255) / 256, step = (blocks + kRangeSample - 1) / kRangeSample;
     k_range_count<<<(blocks + step - 1) / step, 256, 0, s>>>(n, T->ld, T->w, R->rows, R->lanes == 1 ? kTailBatch : virt, step,
-                                                             T->ell_col, T->tptr, T->tcol, lv->iperm, counts + 1);
+                                                             ws == 8 ? 16 : 32, T->ell_col, T->tptr, T->tcol, lv->iperm,
+                                                             lv->level, counts + 1);
     count_launch(3);
     unsigned long long h[kCounts] = {};
     if (cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -2365,6 +2383,12 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     // threads: 16 warps hold a few levels of a part's chunks; a factor too large for the caches needs its rows
     // loaded further ahead (L+U apply with 512 / 1024 threads: 64 x 64 grid FP32 57.8 / 70.5 us; FP64: 400 x 300
     // 409 / 506, 1000 x 1000 1187 / 1488, 64^3 172 / 195, 100^3 392 / 359, 128^3 543 / 486)
+    // Padding: the rows of a level in a range are a fixed step apart (nx - 1 for a 7-point grid of lines of nx), so at nx = 33,
+    // 65, 97, 129 ... the words of a chunk lie in one bank and every poll of them is as many reads as lanes.  L+U apply
+    // without / with padding, FP64 (FP32): 7-point 33^3 210 / 96 us (190 / 73), 97^3 976 / 359 (907 / 278), 129^3 1116 / 544
+    // (991 / 431); lines of 512 and 1024 need the second term of range_slot.  Steps of about 31 words would suffer from the padding
+    // instead (nx = 32), so the rows decide.
+    R->pad = h[7] < h[6] && (size_t)range_slot(R->rows, 1) * ws <= kRangeSmem ? 1 : 0;
     const long long nnz_bound = (long long)T->w * n + T->tail_nnz;
     const int seg_rows = n / (int)std::max(1ull, h[0]);
     R->threads = R->lanes == 1 && T->w <= 4 && seg_rows >= 40 && avg >= 2000 ? 1024 : 512;
@@ -2385,7 +2409,7 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     const bool slow = (double)h[4] * 10.0 * 2.1 * 4.0 > (double)p->wait_cycles;
     const bool pays = (long long)h[1] * step * 10 <= entries * 8 && h[4] * (streams ? 150 : 100) <= h[5] * 85;
     if (slow || !(pays || forced) ||
-        max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)R->rows * ws) * sms < R->nparts) {
+        max_coop_blocks(range_kernel(T, virt), R->threads, (size_t)range_slot(R->rows, R->pad) * ws) * sms < R->nparts) {
         free_range(R);
         return done(HEC_OK);
     }
@@ -2398,8 +2422,8 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     if (cudaMemsetAsync(R->state, 0, 2 * sizeof(int), s) != cudaSuccess) return done(cuda_error(cudaGetLastError(), "memset"));
     k_range_chunks<<<R->nparts, kRangeTableThreads, 0, s>>>(n, nlev, R->nparts, R->rows, rpw, lv->uplo, lv->iperm, lv->level_ptr,
                                                             total, R->chunks, R->part_chunk);
-    k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, T->ell_col, T->tptr, T->tcol, lv->iperm,
-                                                     R->ell_col, R->tcol);
+    k_range_cols<<<(T->ld + 255) / 256, 256, 0, s>>>(n, T->ld, T->w, R->rows, R->pad, T->ell_col, T->tptr, T->tcol,
+                                                     lv->iperm, R->ell_col, R->tcol);
     const int fb = std::min(4096, (n + 255) / 256);  // the words of the first sweep; each sweep sets its successor's
     if (ws == 8) k_fill_sentinel<double><<<fb, 256, 0, s>>>((double*)R->xpb[0], n);
     else k_fill_sentinel<float><<<fb, 256, 0, s>>>((float*)R->xpb[0], n);

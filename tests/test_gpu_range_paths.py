@@ -39,6 +39,11 @@ def test_declined_plan_builds_no_tables():
 
 PATHS = {  # name: (L and U, slab width)
     **{name: (lambda hec, make=make, k=k: hec.ilu_factor(*dev(make()), k=k), w) for name, (make, k, w) in FACTORS.items()},
+    "lines_97": (lambda hec: hec.ilu_factor(*dev(_box(97, 20, 23)), k=0), -1),   # a level's rows 96 apart: padded words
+    "lines_32": (lambda hec: hec.ilu_factor(*dev(_box(32, 40, 23)), k=0), -1),   # 31 apart: padding would collide
+    "plane_513": (lambda hec: hec.ilu_factor(*dev(synth.poisson2d_5pt(513, 90)), k=0), -1),
+    "plane_65": (lambda hec: hec.ilu_factor(*dev(synth.poisson2d_5pt(65, 190)), k=0), -1),
+    "27pt_34": (lambda hec: hec.ilu_factor(*dev(synth.stencil27_jitter(34, seed=3)), k=0), -1),  # two lanes a row, 32 apart
     "box_w4": (lambda hec: hec.ilu_factor(*dev(_box(19, 23, 17)), k=0), 4),
     "ilut_w8": (lambda hec: hec.ilut_factor(*dev(_box(19, 23, 17)), p=10, tol=1e-4), 8),  # four partial sums, two slots a wait
 }

@@ -108,3 +108,17 @@ def test_default_schedule_is_not_the_slower_one(case):
     default, two = (hec.IluSolver(L, U, vdt=vdt, max_nrhs=k) for k in (1, 2))
     t1, t2 = fastest([lambda: default.apply(b), lambda: two.apply(b)])
     assert t1 <= 1.1 * t2, (t1, t2)
+
+
+@pytest.mark.parametrize("nx", [65, 97])
+def test_range_words_out_of_one_bank(nx):
+    """Lines of 64 k + 1 or 96 + 1 points: the rows of a level lie 64 or 96 words apart in a range's shared solution, one bank without
+    padding (97 x 76 x 83, FP64, L+U apply 900 us; the global schedule 520, with padding 290)."""
+    from paper_1606_00541_gb300 import hec
+    n = nx * 76 * 83
+    A = synth.fv7_lognormal_box(nx, 76, 83, np.ones(n))
+    L, U = [h.tensors() for h in hec.ilu_factor(*dev(A), k=0)]
+    b = torch.ones(n, dtype=torch.float64, device="cuda")
+    default, two = (hec.IluSolver(L, U, max_nrhs=k) for k in (1, 2))
+    t1, t2 = fastest([lambda: default.apply(b), lambda: two.apply(b)])
+    assert t1 <= 0.9 * t2, (t1, t2)
