@@ -2151,8 +2151,8 @@ hec_status build_partition(sptrsv_plan* p, const int* part, int nparts, cudaStre
 namespace {
 // what the choice needs to know of the columns: counts[0] += entries whose row is in another range, counts[1] +=
 // the longest tail (without the diagonal) of each 32 rows, in waits of `batch` entries, counts[2] += how many 32
-// rows have a tail, counts[5] and counts[6] += for each row, the rows of its chunk whose word is in the same bank of
-// the shared solution, without and with padding (banks: of 8-byte words 16, of 4-byte words 32).  Of every `step`-th
+// rows have a tail, counts[5] and counts[6] += the most rows of one chunk in one bank of the shared solution, without
+// and with padding (32 banks of 4-byte words, 16 of 8-byte words, whose reads go by half warps).  Of every `step`-th
 // 256 rows of the level order: the choices need shares, not totals, and 256 K rows give them
 constexpr int kRangeSample = 1024;
 __global__ void k_range_count(int n, int ld, int w, int rows, int batch, int step, int banks, const int* __restrict__ ec,
@@ -2177,10 +2177,11 @@ __global__ void k_range_count(int n, int ld, int w, int rows, int batch, int ste
     }
     cross = __reduce_add_sync(0xffffffffu, cross);
     waits = __reduce_max_sync(0xffffffffu, waits);
-    const unsigned same = __match_any_sync(0xffffffffu, chunk);
+    const unsigned together = banks == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
+    const unsigned same = __match_any_sync(0xffffffffu, chunk) & together;
     const int c0 = __popc(same & __match_any_sync(0xffffffffu, word % banks));
     const int c1 = __popc(same & __match_any_sync(0xffffffffu, range_slot(word, 1) % banks));
-    const int plain = __reduce_add_sync(0xffffffffu, c0), padded = __reduce_add_sync(0xffffffffu, c1);
+    const int plain = __reduce_max_sync(0xffffffffu, c0), padded = __reduce_max_sync(0xffffffffu, c1);
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(counts + 5, (unsigned long long)plain);
         atomicAdd(counts + 6, (unsigned long long)padded);
@@ -2387,8 +2388,9 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     // 65, 97, 129 ... the words of a chunk lie in one bank and every poll of them is as many reads as lanes.  L+U apply
     // without / with padding, FP64 (FP32): 7-point 33^3 210 / 96 us (190 / 73), 97^3 976 / 359 (907 / 278), 129^3 1116 / 544
     // (991 / 431); lines of 512 and 1024 need the second term of range_slot.  Steps of about 31 words would suffer from the padding
-    // instead (nx = 32), so the rows decide.
-    R->pad = h[7] < h[6] && (size_t)range_slot(R->rows, 1) * ws <= kRangeSmem ? 1 : 0;
+    // instead (nx = 32), and for a conflict of two the uneven steps of the padding are no gain (9-point 400 x 400 FP64 1148 /
+    // 1384 us), so the rows decide.
+    R->pad = h[7] * 10 < h[6] * 7 && (size_t)range_slot(R->rows, 1) * ws <= kRangeSmem ? 1 : 0;
     const long long nnz_bound = (long long)T->w * n + T->tail_nnz;
     const int seg_rows = n / (int)std::max(1ull, h[0]);
     R->threads = R->lanes == 1 && T->w <= 4 && seg_rows >= 40 && avg >= 2000 ? 1024 : 512;
