@@ -2397,14 +2397,17 @@ hec_status build_range(sptrsv_plan* p, bool forced) {
     const long long entries = nnz_bound - n;  // off-diagonals and padding
     // rows of more than four slots are not loaded a chunk ahead: a factor too large to stay in L2 then shows the
     // latency of its loads (27-point ILU(0) on 100^3: 2116 us against 2086 for the global kernel, ILUT BF16 2100 / 1710)
+    // (a level of a few rows has its loads far ahead: ILUT of the 7-point 12 x 12 x 6000, FP32, global / ranges 74.9 / 64.7 ms)
     const bool streams =
-        (R->lanes > 1 || T->w > 4) &&
+        (R->lanes > 1 ? avg >= 400 : T->w > 4) &&
         (double)(R->lanes > 1 ? nnz_bound : (long long)T->w * n) * (4 + (T->vdt == HEC_BF16 ? 2 : ws)) > (R->lanes > 1 ? 65e6 : 75e6);
-    // rows with a tail wait once for each V entries of the chunk's longest (see the kernel), 0.35 us each beyond the
-    // first, where the global kernel takes 2 V entries together with the slab's; the chain runs through such rows
-    // (red-black 7-point 100^3, ILU(1) and ILUT, FP32, L+U apply with ranges / global: 1193 / 823, 1637 / 1288 us)
+    // rows with a tail wait once for each V entries of the chunk's longest (see the kernel), where the global kernel
+    // takes 2 V entries together with the slab's; the chain runs through such rows.  A wait beyond the first is short when
+    // its words are in the range and an L2 round trip when they are not (red-black 7-point 100^3, ILU(1) and ILUT,
+    // FP32, L+U apply with ranges / global: 1193 / 823, 1637 / 1288 us; dense blocks of 48 rows, none in another range: 59 / 96)
     const double tail_waits = R->lanes > 1 ? (double)h[2] / (double)std::max(1ull, h[3]) : 0.0;
-    h[4] += (unsigned long long)(35.0 * std::max(0.0, tail_waits - 1.0) * nlev);
+    const double away = (double)h[1] * step / (double)std::max(1LL, entries);
+    h[4] += (unsigned long long)((7.0 + 45.0 * away) * std::max(0.0, tail_waits - 1.0) * nlev);
     // the last range waits from the start of the sweep for the chain to reach it, where a warp of the global
     // kernel only waits for the chunks in flight before its own: its wait must stay well inside the budget
     // (four times the estimated sweep at 2.1 GHz)

@@ -83,3 +83,20 @@ def test_unpublished_row_ends_the_waits(case):
     assert hec.hec_sync_status(bad) == hec.STATUS_NAMES.index("TIMEOUT")
     good, ref = (hec.sptrsv_plan_create(H, lv, schedule=s) for s in ("range", "global"))
     assert torch.equal(hec.sptrsv_lower(good, b), hec.sptrsv_lower(ref, b))
+
+
+def test_dense_blocks_take_the_ranges():
+    """Blocks of 48 rows, all entries beyond the slab in the row's own range: the long tails are short waits there."""
+    from paper_1606_00541_gb300 import hec
+    m, b = 500, 48
+    n = m * b
+    rp = np.arange(n + 1, dtype=np.int32) * b
+    ci = (np.arange(n)[:, None] // b * b + np.arange(b)).astype(np.int32).ravel()
+    v = synth._rng(1).uniform(-1.0, 1.0, n * b)
+    v[ci == np.repeat(np.arange(n), b)] = 1.5 * b
+    T = hec.ilu_factor(*dev((rp, ci, v)), k=0)[0].tensors()
+    H, lv = packed(hec, T, 0)
+    plan, ref = hec.sptrsv_plan_create(H, lv), hec.sptrsv_plan_create(H, lv, schedule="global")
+    x = torch.ones(n, dtype=torch.float64, device="cuda")
+    (ran, y), (_, z) = (launches(hec, lambda: hec.sptrsv_lower(p, x)) for p in (plan, ref))
+    assert ran == 1 and torch.equal(y, z)
